@@ -130,12 +130,13 @@ int bp_decode_workspace_size(const pc_code* code, int64_t B, size_t* bytes);
  *     residue (always 1 when crc_len == 0).
  *   d_workspace: bp_decode_workspace_size bytes, overwritten.
  * Messages are FP32; every FP32 operation is rounded as written (no fused
- * multiply-add), so results are reproducible bit for bit.  N >= 128 runs the
- * kernel that keeps each stage group's interior messages in tensor memory
- * (groups of 2 stages up to N = 256, of 3 from 512), smaller N the shared-memory
- * stage-grouped kernel (the environment variable
- * PCBP_DECODER=grouped selects the latter for every N; the outputs are the
- * same).  The frames of a call share a persistent grid: each CTA holds one
+ * multiply-add), so results are reproducible bit for bit.  Scaled min-sum at
+ * every N and exact box-plus below N = 128 run the kernel that keeps a frame's
+ * messages in registers; exact box-plus from N = 128 on runs the kernel that
+ * keeps each stage group's interior messages in tensor memory (groups of 2
+ * stages up to N = 256, of 3 from 512).  The environment variable PCBP_DECODER
+ * selects the latter for every f (tmem, N >= 128) or the shared-memory
+ * stage-grouped kernel (grouped); the outputs are the same.  The frames of a call share a persistent grid: each CTA holds one
  * frame per slot and fetches the next frame index from d_workspace. */
 int bp_decode(const pc_code* code, const float* d_llr, const pc_sched* sched,
               int32_t max_iters, int64_t B, uint32_t* d_bits, int32_t* d_iters,
@@ -270,8 +271,8 @@ typedef struct {
     pc_sched sched;           /* frame b draws events with frame id sched.frame_base + b */
     int32_t max_iters;
     int32_t slots;            /* frames resident per CTA; 0 = as many as fit */
-    int32_t threads_per_frame;/* 0: the bp_decode kernel for this N; otherwise the count of one
-                                 kernel as bp_kernel_threads reports it (TMEM-resident stage
+    int32_t threads_per_frame;/* 0: the bp_decode kernel for this N; otherwise the count of one of
+                                 the other two kernels as bp_kernel_threads reports it (TMEM-resident stage
                                  groups: N/4 for N = 128..512, N/8 for 1024 and 2048;
                                  shared-memory groups: max(32, N/4)); anything else is
                                  PC_EUNSUPPORTED */
@@ -305,7 +306,7 @@ int pc_build_info(int32_t* flags);
  * with TMEM-resident stage groups, N = 128..2048, groups of 2 stages up to
  * N = 256 and of 3 from N = 512, so N/4 or N/8; kernel 1: the shared-memory
  * stage-grouped kernel, max(32, N/4)), the value pc_batch.threads_per_frame
- * takes to select it; where the two are equal the TMEM kernel runs unless
+ * takes to select it (0 selects the kernel bp_decode runs); where the two are equal the TMEM kernel runs unless
  * PCBP_DECODER=grouped.  Host only, no device call.  No counterpart in the
  * paper.  PC_EUNSUPPORTED when the kernel has no build for N. */
 int bp_kernel_threads(const pc_code* code, int32_t kernel, int32_t* threads_per_frame);

@@ -70,6 +70,10 @@ def _jobs() -> list[tuple[Path, Path, list[str]]]:
         extra = [f"-DPCBP_KB3={int(kb3)}"] if use else []
         jobs.append((obj, CSRC / "bp_inst3.cu", [*common, f"-DPCBP_LOGN={n}", *extra, "-c",
                                                  str(CSRC / "bp_inst3.cu"), "-o", str(obj)]))
+    for n in LOGNS:
+        obj = BUILD / f"bp_inst4_{n}.o"
+        jobs.append((obj, CSRC / "bp_inst4.cu", [*common, f"-DPCBP_LOGN={n}", "-c", str(CSRC / "bp_inst4.cu"),
+                                                 "-o", str(obj)]))
     for name in ("bp_decode.cu", "bp_decode_static.cu", "bp_selfcheck.cu", "wbp.cu"):
         obj = BUILD / (Path(name).stem + ".o")
         jobs.append((obj, CSRC / name, [*common, "-c", str(CSRC / name), "-o", str(obj)]))

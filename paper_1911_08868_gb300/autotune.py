@@ -4,9 +4,10 @@ frame (which decoder kernel) and frames resident per CTA ("slots").
 For each length it decodes a synthetic batch (rate 1/2, BPSK/AWGN at the given
 Eb/N0, the given schedule) with every candidate shape through a single-batch
 MixedDecoder, times the launches with CUDA events and keeps the fastest.
-Threads per frame: the counts bp_kernel_threads reports for the two kernels
-(TMEM-resident stage groups: N/4 up to N = 256, N/8 from 512; shared-memory
-groups: max(32, N/4); where they coincide the library runs the TMEM kernel).  Results are cached per GPU
+Threads per frame: 0 (the kernel bp_decode runs) and the counts bp_kernel_threads
+reports for the two others (TMEM-resident stage groups: N/4 up to N = 256, N/8 from
+512; shared-memory groups: max(32, N/4); where they coincide the library runs the
+TMEM kernel).  Results are cached per GPU
 name, library build and schedule in a JSON file ($PCBP_TUNE_CACHE, default ~/.cache/pcbp_tune.json).
 """
 from __future__ import annotations
@@ -30,9 +31,10 @@ def crc_for(N: int):
 
 
 def threads_candidates(pcbp, code):
-    """Distinct threads-per-frame counts that select a decoder kernel for this code (where both
-    kernels take the same count, the library runs the TMEM one)."""
-    return sorted({t for t in (pcbp.bp_kernel_threads(code, k) for k in (0, 1)) if t})
+    """Distinct threads-per-frame counts that select a decoder kernel for this code: 0 (bp_decode's)
+    and those of the two kernels that have a count of their own (where both take the same one, the
+    library runs the TMEM kernel)."""
+    return [0, *sorted({t for t in (pcbp.bp_kernel_threads(code, k) for k in (0, 1)) if t})]
 
 
 def _synthetic(pcbp, inputs, dev, N, K, r, poly, B, ebn0, seed):

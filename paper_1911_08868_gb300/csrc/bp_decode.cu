@@ -208,6 +208,45 @@ bool tmem_for(int n, int N, int tpf)
     return tpf != std::max(32, N / 4) || use_tmem_kernel(n);
 }
 
+// The decoder kernels (PCBP_DECODER=grouped or =tmem keeps to one of the older two).
+enum Kernel { kGrouped = 0, kTmem = 1, kWarp = 2 };
+
+void shape4_of(int n, int K, int slots, int* max_slots, size_t* smem)
+{
+#define PCBP_SHAPE4(k) bp4_shape_##k(K, slots, max_slots, smem)
+    PCBP_SWITCH_N(n, PCBP_SHAPE4)
+#undef PCBP_SHAPE4
+}
+
+int occupancy4_of(int n, const LaunchGeom& g, int fk)
+{
+    int occ = 0;
+#define PCBP_OCC4(k) occ = bp4_occupancy_##k(g, fk)
+    PCBP_SWITCH_N(n, PCBP_OCC4)
+#undef PCBP_OCC4
+    return occ;
+}
+
+cudaError_t launch4_of(int n, const WarpParams& P, const LaunchGeom& g, int fk, cudaStream_t st, bool pdl)
+{
+    cudaError_t e = cudaSuccess;
+#define PCBP_LAUNCH4(k) e = bp4_launch_##k(P, g, fk, st, pdl)
+    PCBP_SWITCH_N(n, PCBP_LAUNCH4)
+#undef PCBP_LAUNCH4
+    return e;
+}
+
+// The kernel of a batch that asks for tpf threads per frame (0: the decoder's choice, the
+// register-resident kernel where it is built).
+Kernel kernel_for(int n, int N, int tpf, int fk)
+{
+    if (tpf != 0) return tmem_for(n, N, tpf) ? kTmem : kGrouped;
+    const char* v = std::getenv("PCBP_DECODER");
+    if (v && std::strcmp(v, "grouped") == 0) return kGrouped;
+    if (n >= 7 && v && std::strcmp(v, "tmem") == 0) return kTmem;
+    return warp_kernel_has(n, fk) ? kWarp : kTmem;
+}
+
 size_t table_bytes(int N, int r, int K)
 {
     const size_t nw = size_t(N >= 32 ? N / 32 : 1);
@@ -293,6 +332,31 @@ int plan_launch3(const pc_code* c, int64_t B, int fk, LaunchGeom* g, int slots_r
     return PC_OK;
 }
 
+// Register-resident kernel: as many frames per CTA as it is built for; where the batch does not
+// fill the chip, fewer frames per CTA on more SMs (a frame alone on its SM takes about half the
+// time per iteration of one that shares it).
+int plan_launch4(const pc_code* c, int64_t B, int fk, LaunchGeom* g, int slots_req = 0)
+{
+    DeviceInfo di;
+    int rc = device_info(&di);
+    if (rc != PC_OK) return rc;
+    int slots = 0;
+    size_t smem = 0;
+    shape4_of(c->n, c->K, 1, &slots, &smem);
+    if (slots_req > 0) slots = std::min(slots, slots_req);
+    slots = int(std::max<int64_t>(1, std::min<int64_t>(slots, (B + di.sms - 1) / di.sms)));
+    int max_slots = 0;
+    shape4_of(c->n, c->K, slots, &max_slots, &smem);
+    if (smem > size_t(di.smem_optin)) return PC_EUNSUPPORTED;
+    g->slots = slots;
+    g->smem = smem;
+    g->grid = 1;
+    const int occ = occupancy4_of(c->n, *g, fk);
+    if (occ < 1) return PC_EUNSUPPORTED;
+    g->grid = int(std::min<int64_t>((B + slots - 1) / slots, int64_t(di.sms) * occ));
+    return PC_OK;
+}
+
 int validate_events(const pc_code* c, const pc_event* ev, int n_ev)
 {
     if (n_ev < 0 || n_ev > PC_MAX_EVENTS) return PC_EINVAL;
@@ -311,6 +375,22 @@ int validate_events(const pc_code* c, const pc_event* ev, int n_ev)
     return PC_OK;
 }
 
+// The batch's buffers and schedule as every decoder kernel reads them.
+void fill_job(const pc_code* code, const float* d_llr, const pc_sched* sched, int32_t max_iters, int64_t B,
+              uint32_t* d_bits, int32_t* d_iters, uint8_t* d_crc_ok, FrameJob* job)
+{
+    build_dev_sched(sched, &job->S);
+    job->llr = d_llr;
+    job->bits = d_bits;
+    job->iters = d_iters;
+    job->crc_ok = d_crc_ok;
+    job->B = B;
+    job->max_iters = max_iters;
+    job->K = code->K;
+    job->r = code->crc_len;
+    job->neg_zero = -0.0f;
+}
+
 // Kernel parameters of one batch (no device calls).
 void fill_params(const pc_code* code, const float* d_llr, const pc_sched* sched, int32_t max_iters, int64_t B,
                  uint32_t* d_bits, int32_t* d_iters, uint8_t* d_crc_ok, BpParams* P)
@@ -324,16 +404,15 @@ void fill_params(const pc_code* code, const float* d_llr, const pc_sched* sched,
     P->crc_ok = d_crc_ok;
     P->B = B;
     P->max_iters = max_iters;
-    P->job.S = P->sched;
-    P->job.llr = d_llr;
-    P->job.bits = d_bits;
-    P->job.iters = d_iters;
-    P->job.crc_ok = d_crc_ok;
-    P->job.B = B;
-    P->job.max_iters = max_iters;
-    P->job.K = code->K;
-    P->job.r = code->crc_len;
-    P->job.neg_zero = -0.0f;
+    fill_job(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, &P->job);
+}
+
+void fill_warp_params(const pc_code* code, const float* d_llr, const pc_sched* sched, int32_t max_iters, int64_t B,
+                      uint32_t* d_bits, int32_t* d_iters, uint8_t* d_crc_ok, WarpParams* P)
+{
+    std::memset(P, 0, sizeof(WarpParams));
+    fill_job(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, &P->job);
+    build_warp_code(code, P);
 }
 
 // d_post (posterior output, nullable): the TMEM kernel's debug build that also writes L at node
@@ -362,6 +441,19 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
             if (rc != PC_OK) return rc;
         }
     }
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    LaunchGeom g;
+    const Kernel kind = d_post ? kTmem : kernel_for(code->n, code->N, 0, sched->fkind);
+    if (!trace && kind == kWarp) {
+        std::unique_ptr<WarpParams> W(new WarpParams);
+        fill_warp_params(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, W.get());
+        rc = plan_launch4(code, B, sched->fkind, &g);
+        if (rc != PC_OK) return rc;
+        W->slots = g.slots;
+        W->counter = reinterpret_cast<unsigned long long*>(d_workspace);
+        if (cudaMemsetAsync(d_workspace, 0, 32, st) != cudaSuccess) return PC_ECUDA;
+        return launch4_of(code->n, *W, g, sched->fkind, st, false) == cudaSuccess ? PC_OK : PC_ECUDA;
+    }
     std::unique_ptr<BpParams> P(new BpParams);
     fill_params(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, P.get());
     if (trace && h_events) {
@@ -379,13 +471,11 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
 
     P->job.post = d_post;
 
-    LaunchGeom g;
-    const bool tmem = !trace && (d_post || use_tmem_kernel(code->n));
+    const bool tmem = !trace && kind == kTmem;
     rc = trace ? plan_launch(code, B, trace, sched->fkind, &g)
                : (tmem ? plan_launch3(code, B, sched->fkind, &g) : plan_launch2(code, B, sched->fkind, &g));
     if (rc != PC_OK) return rc;
     P->slots = g.slots;
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
 #ifdef PCBP_CHECKED
     // bound-check status word at byte 16 of the workspace (read back by the caller)
     P->job.check = reinterpret_cast<unsigned*>(static_cast<unsigned char*>(d_workspace) + 16);
@@ -564,9 +654,13 @@ namespace {
 constexpr uint32_t kMixedMagic = 0x70636278u;
 
 struct MixedEntry {
-    BpParams P;
+    union {
+        BpParams P;        // kGrouped, kTmem
+        WarpParams W;      // kWarp
+    };
+    int64_t B;
     LaunchGeom g;
-    int32_t n, tmem, fkind;
+    int32_t n, kernel, fkind;
     uint32_t magic;
 };
 
@@ -611,16 +705,23 @@ extern "C" int bp_mixed_prepare(const pc_batch* batches, int32_t n_batches, void
         const pc_batch& b = batches[i];
         std::unique_ptr<MixedEntry> m(new MixedEntry);
         std::memset(m.get(), 0, sizeof(MixedEntry));
-        fill_params(b.code, b.d_llr, &b.sched, b.max_iters, b.B, b.d_bits, b.d_iters, b.d_crc_ok, &m->P);
         m->n = b.code->n;
         m->fkind = b.sched.fkind;
-        const int tpf = b.threads_per_frame;
-        m->tmem = tmem_for(b.code->n, b.code->N, tpf) ? 1 : 0;
+        m->B = b.B;
         if (b.B > 0) {
-            const int rc = m->tmem ? plan_launch3(b.code, b.B, b.sched.fkind, &m->g, b.slots)
-                                   : plan_launch2(b.code, b.B, b.sched.fkind, &m->g, b.slots);
+            const Kernel kind = kernel_for(b.code->n, b.code->N, b.threads_per_frame, b.sched.fkind);
+            m->kernel = kind;
+            const int rc = kind == kWarp   ? plan_launch4(b.code, b.B, b.sched.fkind, &m->g, b.slots)
+                 : kind == kTmem ? plan_launch3(b.code, b.B, b.sched.fkind, &m->g, b.slots)
+                                 : plan_launch2(b.code, b.B, b.sched.fkind, &m->g, b.slots);
             if (rc != PC_OK) return rc;
-            m->P.slots = m->g.slots;
+            if (kind == kWarp) {
+                fill_warp_params(b.code, b.d_llr, &b.sched, b.max_iters, b.B, b.d_bits, b.d_iters, b.d_crc_ok, &m->W);
+                m->W.slots = m->g.slots;
+            } else {
+                fill_params(b.code, b.d_llr, &b.sched, b.max_iters, b.B, b.d_bits, b.d_iters, b.d_crc_ok, &m->P);
+                m->P.slots = m->g.slots;
+            }
         }
         m->magic = kMixedMagic;
         std::memcpy(static_cast<MixedEntry*>(h_table) + i, m.get(), sizeof(MixedEntry));
@@ -662,9 +763,11 @@ extern "C" int bp_slot_limit(const pc_code* code, int32_t threads_per_frame, int
     if (tpf < 0) return PC_EINVAL;
     if (tpf != 0 && tpf != tmem_threads_per_frame(code->n) && tpf != std::max(32, N / 4))
         return PC_EUNSUPPORTED;
-    const bool tmem = tmem_for(code->n, N, tpf);
     LaunchGeom g;
-    rc = tmem ? plan_launch3(code, 1, fkind, &g) : plan_launch2(code, 1, fkind, &g);
+    const Kernel kind = kernel_for(code->n, N, tpf, fkind);
+    rc = kind == kWarp   ? plan_launch4(code, INT32_MAX, fkind, &g)
+         : kind == kTmem ? plan_launch3(code, 1, fkind, &g)
+                         : plan_launch2(code, 1, fkind, &g);
     if (rc != PC_OK) return rc;
     *max_slots = g.slots;
     return PC_OK;
@@ -695,10 +798,13 @@ extern "C" int bp_decode_mixed(const void* h_table, int32_t n_batches, void* d_w
     bool first = true;
     for (int i = 0; i < n_batches; ++i) {
         std::memcpy(m.get(), static_cast<const MixedEntry*>(h_table) + i, sizeof(MixedEntry));
-        if (m->P.B == 0) continue;
-        m->P.counter = reinterpret_cast<unsigned long long*>(d_workspace) + i;
-        const cudaError_t e = m->tmem ? launch3_of(m->n, m->P, m->g, m->fkind, st, !first)
-                                      : launch2_of(m->n, m->P, m->g, m->fkind, st, !first);
+        if (m->B == 0) continue;
+        unsigned long long* const counter = reinterpret_cast<unsigned long long*>(d_workspace) + i;
+        if (m->kernel == kWarp) m->W.counter = counter;
+        else m->P.counter = counter;
+        const cudaError_t e = m->kernel == kWarp   ? launch4_of(m->n, m->W, m->g, m->fkind, st, !first)
+                              : m->kernel == kTmem ? launch3_of(m->n, m->P, m->g, m->fkind, st, !first)
+                                                   : launch2_of(m->n, m->P, m->g, m->fkind, st, !first);
         if (e != cudaSuccess) return PC_ECUDA;
         first = false;
     }

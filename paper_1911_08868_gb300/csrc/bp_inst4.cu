@@ -1,0 +1,76 @@
+// Instantiates the register-resident decoder kernel for one code length,
+// 2^PCBP_LOGN (compiled once per n = 3..11).
+#include "bp_kernel4.cuh"
+#include "bp_launch.h"
+
+#ifndef PCBP_LOGN
+#error "PCBP_LOGN must be defined"
+#endif
+
+#define PCBP_CAT2(a, b) a##b
+#define PCBP_CAT(a, b) PCBP_CAT2(a, b)
+
+namespace pcbp {
+
+namespace {
+using Geo = G4<PCBP_LOGN>;
+
+// pdl: programmatic dependent launch, the grid may start while the previous
+// kernel of the stream still runs (for independent batches).
+template <int FK, int WG>
+cudaError_t launch_variant(const WarpParams& P, const LaunchGeom& g, cudaStream_t st, bool pdl)
+{
+    auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, WG>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(g.grid));
+    cfg.blockDim = dim3(unsigned(g.slots * 32 * Geo::WPF));
+    cfg.dynamicSmemBytes = g.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, P);
+}
+
+template <int FK>
+int occupancy(const LaunchGeom& g)
+{
+    auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, 0>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) != cudaSuccess)
+        return 0;
+    int blocks = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, g.slots * 32 * Geo::WPF, g.smem) != cudaSuccess)
+        return 0;
+    return blocks;
+}
+}  // namespace
+
+void PCBP_CAT(bp4_shape_, PCBP_LOGN)(int K, int slots, int* max_slots_out, size_t* smem_out)
+{
+    *max_slots_out = Geo::SLOTS;
+    *smem_out = Geo::smem_bytes(K, slots);
+}
+
+int PCBP_CAT(bp4_occupancy_, PCBP_LOGN)(const LaunchGeom& g, int fkind)
+{
+    if (fkind) return warp_kernel_has(PCBP_LOGN, 1) ? occupancy<PCBP_LOGN <= 6 ? 1 : 0>(g) : 0;
+    return occupancy<0>(g);
+}
+
+cudaError_t PCBP_CAT(bp4_launch_, PCBP_LOGN)(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st,
+                                             bool pdl)
+{
+    const bool wg = (P.job.S.stop_kind & 2) != 0;
+    if (fkind) {
+        if (!warp_kernel_has(PCBP_LOGN, 1)) return cudaErrorInvalidValue;
+        constexpr int FK = PCBP_LOGN <= 6 ? 1 : 0;
+        return wg ? launch_variant<FK, 1>(P, g, st, pdl) : launch_variant<FK, 0>(P, g, st, pdl);
+    }
+    return wg ? launch_variant<0, 1>(P, g, st, pdl) : launch_variant<0, 0>(P, g, st, pdl);
+}
+
+}  // namespace pcbp

@@ -1,8 +1,9 @@
 // Per-length launch entry points of the decoder kernels (one set per n):
 // bp_* from bp_inst.cu (per-stage kernel, used for the trace entry), bp2_*
-// from bp_inst2.cu (stage-grouped kernel, bp_decode for n < 7), bp3_* from
+// from bp_inst2.cu (stage-grouped kernel), bp3_* from
 // bp_inst3.cu (stage-grouped kernel with TMEM-resident group interiors,
-// bp_decode for n = 7..11).
+// bp_decode with exact box-plus for n = 7..11), bp4_* from bp_inst4.cu
+// (register-resident kernel, bp_decode otherwise).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -51,5 +52,32 @@ PCBP_DECLARE_LEN3(10)
 PCBP_DECLARE_LEN3(11)
 
 #undef PCBP_DECLARE_LEN3
+
+// Lengths and f the register-resident kernel (bp4_*, bp_inst4.cu) is built for.  Scaled min-sum
+// at every length: against the tensor-memory kernel, time per frame-iteration without an event
+// 0.39 / 0.94 ns (N = 256), 2.18 / 3.47 (1024), 4.89 / 7.48 (2048), under an event 0.51 / 1.16,
+// 3.00 / 3.75 and 7.14 / 8.73.  Exact box-plus below N = 128 only: its f is 8 times as long, and
+// the unrolled iteration no longer fits the instruction cache (N = 256 with events 0.85 times the
+// tensor-memory kernel's speed, N = 128 0.96).
+constexpr bool warp_kernel_has(int n, int fkind) { return n >= 3 && n <= 11 && (fkind == 0 || n <= 6); }
+
+struct WarpParams;
+
+#define PCBP_DECLARE_LEN4(n)                                                                       \
+    void bp4_shape_##n(int K, int slots, int* max_slots_out, size_t* smem_out);                    \
+    int bp4_occupancy_##n(const LaunchGeom& g, int fkind);                                         \
+    cudaError_t bp4_launch_##n(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st, bool pdl);
+
+PCBP_DECLARE_LEN4(3)
+PCBP_DECLARE_LEN4(4)
+PCBP_DECLARE_LEN4(5)
+PCBP_DECLARE_LEN4(6)
+PCBP_DECLARE_LEN4(7)
+PCBP_DECLARE_LEN4(8)
+PCBP_DECLARE_LEN4(9)
+PCBP_DECLARE_LEN4(10)
+PCBP_DECLARE_LEN4(11)
+
+#undef PCBP_DECLARE_LEN4
 
 }  // namespace pcbp

@@ -126,6 +126,20 @@ void build_dev_sched(const pc_sched* s, DevSched* d)
     d->frame_base = s->frame_base;
 }
 
+void build_warp_code(const pc_code* c, WarpParams* p)
+{
+    const int nw = std::max(1, c->N / 32);
+    for (int w = 0; w < nw; ++w) p->frozen[w] = c->frozen_mask[w];
+    if (c->N < 32) p->frozen[0] &= (1u << c->N) - 1u;
+    for (int k = 0; k < c->K; ++k) p->info_idx[k] = (int16_t)c->info_idx[k];
+    uint64_t v = 1;      // x^e mod g, e = K-1-k
+    for (int k = c->K - 1; k >= 0; --k) {
+        p->crc[k] = c->crc_len > 0 ? (uint32_t)v : 0u;
+        v <<= 1;
+        if (c->crc_len > 0 && ((v >> c->crc_len) & 1ull)) v ^= c->crc_poly;
+    }
+}
+
 void build_enc_params(const pc_code* c, EncParams* e)
 {
     std::memset(e, 0, sizeof(EncParams));

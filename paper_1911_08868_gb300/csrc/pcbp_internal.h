@@ -76,6 +76,17 @@ struct BpParams {
     FrameJob job;   // the same batch, as the stage-grouped kernel reads it
 };
 
+// Parameters of the warp-per-frame kernel: the batch and the code as that kernel reads it
+// (crc[k] = x^(K-1-k) mod g of the information bit of rank k).
+struct WarpParams {
+    FrameJob job;
+    unsigned long long* counter;
+    int32_t slots;
+    uint32_t frozen[kMaxWords];
+    uint32_t crc[kMaxN];
+    int16_t info_idx[kMaxN];
+};
+
 // Encoder tables: crc_pay[i] = x^(r + Kp - 1 - i) mod g for payload bit i.
 struct EncParams {
     int32_t N, n, K, r, Kp;
@@ -91,6 +102,7 @@ int validate_code(const pc_code* c);
 int validate_sched(const pc_code* c, const pc_sched* s);
 void build_dev_code(const pc_code* c, DevCode* d);
 void build_dev_sched(const pc_sched* s, DevSched* d);
+void build_warp_code(const pc_code* c, WarpParams* p);
 void build_enc_params(const pc_code* c, EncParams* e);
 uint32_t poly_xpow_mod(int e, int r, uint64_t g);
 
