@@ -1,4 +1,4 @@
-// C-ABI entry points of libpcbp: pc_encode, bp_decode, bp_decode_trace.
+// C-ABI entry points of libpcbp: the decoders (pc_encode is in encode.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -11,14 +11,6 @@
 #include "pcbp_internal.h"
 
 namespace pcbp {
-
-namespace {
-
-struct DeviceInfo {
-    int sms = 0;
-    int smem_optin = 0;
-    int smem_per_sm = 0;
-};
 
 int device_info(DeviceInfo* out)
 {
@@ -39,6 +31,8 @@ int device_info(DeviceInfo* out)
     *out = d;
     return PC_OK;
 }
+
+namespace {
 
 void shape_of(int n, int* T, size_t* slot)
 {
@@ -491,69 +485,11 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
     return PC_OK;
 }
 
-// ---------------------------------------------------------------------------
-// Encoder (Eq. 1): one CTA per frame at a time.  The CRC is the XOR of the
-// per-payload-bit remainders crc_pay[i]; u is built in shared memory and the
-// n butterfly layers x[t] ^= x[t + 2^p] run in place.
-__global__ void __launch_bounds__(256) encode_kernel(const __grid_constant__ EncParams P)
-{
-    extern __shared__ uint8_t su[];
-    __shared__ uint32_t red[8];
-    const int N = P.N, n = P.n, K = P.K, r = P.r, Kp = P.Kp;
-    for (int64_t f = blockIdx.x; f < P.B; f += gridDim.x) {
-        const uint8_t* pay = P.payload + size_t(f) * Kp;
-        uint32_t acc = 0;
-        for (int i = threadIdx.x; i < Kp; i += blockDim.x)
-            if (pay[i] & 1) acc ^= P.crc_pay[i];
-        for (int o = 16; o > 0; o >>= 1) acc ^= __shfl_xor_sync(0xffffffffu, acc, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-        for (int j = threadIdx.x; j < N; j += blockDim.x) su[j] = 0;
-        __syncthreads();
-        uint32_t crc = 0;
-        for (int w = 0; w < int(blockDim.x >> 5); ++w) crc ^= red[w];
-        for (int k = threadIdx.x; k < K; k += blockDim.x) {
-            const uint8_t bit = k < Kp ? uint8_t(pay[k] & 1) : uint8_t((crc >> (r - 1 - (k - Kp))) & 1u);
-            su[P.info_idx[k]] = bit;
-        }
-        __syncthreads();
-        for (int p = 0; p < n; ++p) {
-            for (int q = threadIdx.x; q < N / 2; q += blockDim.x) {
-                const int t = ((q >> p) << (p + 1)) | (q & ((1 << p) - 1));
-                su[t] ^= su[t | (1 << p)];
-            }
-            __syncthreads();
-        }
-        uint8_t* x = P.x + size_t(f) * N;
-        for (int j = threadIdx.x; j < N; j += blockDim.x) x[j] = su[j];
-        __syncthreads();
-    }
-}
-
 }  // namespace
 
 }  // namespace pcbp
 
 using namespace pcbp;
-
-extern "C" int pc_encode(const pc_code* code, const uint8_t* d_payload, uint8_t* d_x, int64_t B, void* stream)
-{
-    int rc = validate_code(code);
-    if (rc != PC_OK) return rc;
-    if (B < 0) return PC_EINVAL;
-    if (B == 0) return PC_OK;
-    if (!d_x || (!d_payload && code->K - code->crc_len > 0)) return PC_EINVAL;
-    DeviceInfo di;
-    rc = device_info(&di);
-    if (rc != PC_OK) return rc;
-    std::unique_ptr<EncParams> P(new EncParams);
-    build_enc_params(code, P.get());
-    P->payload = d_payload;
-    P->x = d_x;
-    P->B = B;
-    const int grid = int(std::min<int64_t>(B, int64_t(di.sms) * 8));
-    encode_kernel<<<grid, 256, size_t(code->N), reinterpret_cast<cudaStream_t>(stream)>>>(*P);
-    return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ECUDA;
-}
 
 extern "C" int bp_decode_workspace_size(const pc_code* code, int64_t B, size_t* bytes)
 {

@@ -148,7 +148,7 @@ void build_enc_params(const pc_code* c, EncParams* e)
     e->K = c->K;
     e->r = c->crc_len;
     e->Kp = c->K - c->crc_len;
-    for (int k = 0; k < c->K; ++k) e->info_idx[k] = (int16_t)c->info_idx[k];
+    for (int w = 0; w < std::max(1, c->N / 32); ++w) e->frozen[w] = c->frozen_mask[w];
     if (c->crc_len > 0) {
         std::vector<uint32_t> pw = xpow_table(c->K, c->crc_len, c->crc_poly);
         for (int i = 0; i < e->Kp; ++i) e->crc_pay[i] = pw[(size_t)(c->K - 1 - i)];

@@ -90,12 +90,20 @@ struct WarpParams {
 // Encoder tables: crc_pay[i] = x^(r + Kp - 1 - i) mod g for payload bit i.
 struct EncParams {
     int32_t N, n, K, r, Kp;
+    uint32_t frozen[kMaxWords];
     uint32_t crc_pay[kMaxN];
-    int16_t info_idx[kMaxN];
     const uint8_t* payload;
     uint8_t* x;
     int64_t B;
 };
+
+// The current device (bp_decode.cu).
+struct DeviceInfo {
+    int sms = 0;
+    int smem_optin = 0;
+    int smem_per_sm = 0;
+};
+int device_info(DeviceInfo* out);
 
 // Host helpers (pcbp_host.cpp).
 int validate_code(const pc_code* c);
