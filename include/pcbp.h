@@ -231,9 +231,9 @@ int wbp_workspace_size(const pc_code* code, int32_t T, int64_t B, int32_t real_b
 int wbp_forward(const pc_code* code, const float* d_llr, const float* d_w, int32_t T, int64_t B,
                 float* d_logits, float* d_ckpt, void* d_workspace, void* stream);
 /* Given d_glogits = dLoss/dlogits [B][K]: d_gw += dLoss/dw (caller zeroes it
- * for a fresh gradient); d_gllr (nullable) = dLoss/dllr [B][N].  Runs one
- * launch per iteration, in reverse, each recomputing its iteration from the
- * checkpoint. */
+ * for a fresh gradient); d_gllr (nullable) = dLoss/dllr [B][N].  Runs the
+ * iterations in reverse, each recomputed from its checkpoint: in one launch for
+ * N <= 1024, else (and in FP64) in one launch per iteration. */
 int wbp_backward(const pc_code* code, const float* d_llr, const float* d_w, int32_t T, int64_t B,
                  const float* d_ckpt, const float* d_glogits, float* d_gw, float* d_gllr,
                  void* d_workspace, void* stream);

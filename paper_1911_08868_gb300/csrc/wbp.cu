@@ -3,9 +3,10 @@
 // each f evaluation has its own learnable scale w[t][s][q][k] (iteration t,
 // stage s, processing element q, and k = 0 L_out1, 1 L_out2, 2 R_out1,
 // 3 R_out2) in place of the fixed min-sum scale.  Forward keeps the R planes
-// at every iteration boundary as checkpoints; backward runs one launch per
-// iteration in reverse, recomputes that iteration from its checkpoint and
-// applies the adjoint of the R sweep then of the L sweep.
+// at every iteration boundary as checkpoints; backward runs the iterations in
+// reverse, recomputes each from its checkpoint and applies the adjoint of the
+// R sweep then of the L sweep (FP32 up to N = 1024 in one launch, else one
+// launch per iteration).
 //
 // Derivatives of f_w(a, b) = w sign(a) sign(b) min(|a|, |b|): with a the
 // minimum (|a| <= |b|: the first operand wins ties), df/da = w sign(b),
@@ -256,16 +257,13 @@ __global__ void __launch_bounds__(1024, 1) wbp_forward_reg_kernel(const __grid_c
     float* L = reinterpret_cast<float*>(smem + tab + size_t(slot) * size_t(2 * n + 1) * N * sizeof(float));
     float* R = L + (n + 1) * N;                   // plane l-2 = level l, 2 <= l <= n+1
     for (int j = tid; j < N; j += tps) R[(n - 1) * N + sw32(j)] = prior_v<float>(s_frozen, j);
-    __shared__ long long s_frame[32];
     const unsigned bid = 1u + unsigned(slot);
     const bool act = tid < NH;                    // N < 64: fewer elements than a warp
     const int q = act ? tid : 0;
 
-    while (true) {
-        if (tid == 0) s_frame[slot] = (long long)atomicAdd(P.counter, 1ull);
-        bar(bid, tps);
-        const long long f = s_frame[slot];
-        if (f >= P.B) break;
+    // every frame takes the same time: a fixed share of the frames per slot, no frame counter
+    const int slots = blockDim.x / tps;
+    for (int64_t f = int64_t(blockIdx.x) * slots + slot; f < P.B; f += int64_t(gridDim.x) * slots) {
         copy_async_sw(L, P.llr + size_t(f) * N, N, tid, tps);
         for (int j = tid; j < (n - 1) * N; j += tps) R[j] = 0.f;
         if (P.ckpt)
@@ -573,8 +571,7 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
     constexpr int NW = N >= 32 ? N / 32 : 1;
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = P.code.K;
-    const int tps = P.tps, it = P.it;
-    const bool last = it == P.T - 1;
+    const int tps = P.tps;
     uint32_t* s_frozen = reinterpret_cast<uint32_t*>(smem);
     int16_t* s_info = reinterpret_cast<int16_t*>(s_frozen + NW);
     const size_t tab = (size_t(NW) * 4 + size_t(K) * 2 + 15) & ~size_t(15);
@@ -593,11 +590,16 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
     float* const Rck = G + (n - 1) * N;                                                 // R(it), levels 2..n
     for (int j = tid; j < N; j += tps) Pri[sw32(j)] = prior_v<float>(s_frozen, j);
     for (int j = tid; j < (n + 1) * N; j += tps) gL[j] = 0.f;
-    __shared__ long long s_frame[32], s_next[32];
     const unsigned bid = 1u + unsigned(slot);
-    const float* wt = P.w + size_t(it) * n * NH * 4;
+    const int slots = blockDim.x / tps;
     const bool act = tid < NH;                 // N < 64: fewer elements than a warp
     const int q = act ? tid : 0;
+    // One launch runs the iterations in reverse, with a fixed share of the frames in each slot (the
+    // gradient of R(t) that a frame leaves is read again by the same slot only): no launch, counter
+    // and drain between iterations.  Forth and back over the frames, so that an iteration starts with
+    // the gradients written last, which L2 still holds.
+    for (int it = P.T - 1; it >= 0; --it) {
+    const bool last = it == P.T - 1;
     float dwr[n][4];
 #pragma unroll
     for (int s = 0; s < n; ++s)
@@ -607,26 +609,28 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
     // the thread's weight pairs of this iteration, each loaded one stage ahead of its use (the
     // weights are read-only and the same for every frame of the launch, so a load may be issued
     // before the barrier that ends the stage using the previous pair): w[k], w[k+1] of stage s
+    const float* wt = P.w + size_t(it) * n * NH * 4;
     auto wpair = [&](int s, int k) { return ld_pair(wt + (s * NH + q) * 4 + k); };
-    // inputs of frame fx: the checkpoint R(it), the LLRs (L level 1) and (before the last
-    // iteration) the incoming gradient
-    auto fetch = [&](long long fx) {
-        copy_async(Rck, P.ckpt + (size_t(it) * P.B + size_t(fx)) * (n - 1) * N, (n - 1) * N, tid, tps);
-        copy_async_sw(L, P.llr + size_t(fx) * N, N, tid, tps);
-        if (!last) copy_async(G, P.gin + size_t(fx) * (n - 1) * N, (n - 1) * N, tid, tps);
-    };
-    // the next frame's index is taken as a frame starts and published by the slot leader a few
-    // stages later, before the slot barrier that ends the last forward stage of distance 2^6 or
-    // more (or the first stage, where the slot is one warp), so the atomic's round trip overlaps
-    // the stages
-    constexpr int s_pub = n >= 7 ? n - 7 : 0;
     float2 wc = wpair(0, 0);
-    if (tid == 0) s_frame[slot] = (long long)atomicAdd(P.counter, 1ull);
-    bar(bid, tps);
-    long long f = s_frame[slot];
-    while (f < P.B) {
-        unsigned long long nf = 0;
-        if (tid == 0) nf = atomicAdd(P.counter, 1ull);
+    // (32-bit frame numbers: the checkpoints and gradient states of 2^31 frames exceed any memory)
+    const bool back = (P.T - 1 - it) & 1;
+    const int f0 = int(blockIdx.x) * slots + slot, fs = int(gridDim.x) * slots;
+    int left = f0 < P.B ? (int(P.B) - 1 - f0) / fs + 1 : 0;
+    const int f_step = back ? -fs : fs;
+    for (int f = back ? f0 + fs * (left - 1) : f0; left > 0; --left, f += f_step) {
+        // the buffers' addresses from a copy of `it` the compiler cannot see through: held across the
+        // frames they would take six of the 128 registers (backward 5% slower at N = 1024)
+        int iv = it;
+        asm volatile("" : "+r"(iv));
+        wt = P.w + size_t(iv) * n * NH * 4;
+        float* gout = P.gout + (size_t((P.T - iv) & 1) * P.B + size_t(f)) * (n - 1) * N;
+        // inputs of the frame: the checkpoint R(it), the LLRs (L level 1) and (before the last
+        // iteration) the incoming gradient, written by iteration it+1
+        auto fetch = [&](int fx) {
+            copy_async(Rck, P.ckpt + (size_t(iv) * P.B + size_t(fx)) * (n - 1) * N, (n - 1) * N, tid, tps);
+            copy_async_sw(L, P.llr + size_t(fx) * N, N, tid, tps);
+            if (!last) copy_async(G, P.gin + (size_t((P.T - 1 - iv) & 1) * P.B + size_t(fx)) * (n - 1) * N, (n - 1) * N, tid, tps);
+        };
         fetch(f);
         copy_wait();
         bar(bid, tps);
@@ -645,13 +649,11 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
                 Lo[t] = fw(lt, radd(lb, rb), w2.x);
                 Lo[b] = radd(fw(rt, lt, w2.y), lb);
             }
-            if (s == s_pub && tid == 0) s_next[slot] = (long long)nf;
             stage_sync(p, p - 1, bid, tps);
         }
-        const long long fn = s_next[slot];
         // this frame's accumulated LLR gradient, read now and added after the adjoint of the L sweep
         float gll[2] = {0.f, 0.f};
-        if (P.gllr) {
+        if (P.gllr && !last) {
 #pragma unroll
             for (int h = 0; h < 2; ++h)
                 if (tid + h * tps < N) gll[h] = P.gllr[size_t(f) * N + tid + h * tps];
@@ -732,7 +734,6 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
             }
         }
         // adjoint of the L sweep: stage s makes L level s+2 from L level s+1 and R(it) level s+2
-        float* gout = P.gout + size_t(f) * (n - 1) * N;
 #pragma unroll
         for (int s = n - 1; s >= 0; --s) {
             const float2 w2 = wc;
@@ -794,15 +795,26 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
                 gL[sw32(j)] = 0.f;
             }
         }
-        f = fn;
     }
     if (act) {
         float* g = P.gw + size_t(it) * n * NH * 4 + size_t(q) * 4;
+        // an element's four values in one reduction where gw allows it
+        const bool vec = (reinterpret_cast<uintptr_t>(P.gw) & 15u) == 0;
 #pragma unroll
-        for (int s = 0; s < n; ++s)
+        for (int s = 0; s < n; ++s) {
+            float* d = g + size_t(s) * NH * 4;
+            if (vec) {
+                if (dwr[s][0] != 0.f || dwr[s][1] != 0.f || dwr[s][2] != 0.f || dwr[s][3] != 0.f)
+                    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(d)),
+                                 "f"(dwr[s][0]), "f"(dwr[s][1]), "f"(dwr[s][2]), "f"(dwr[s][3])
+                                 : "memory");
+            } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (dwr[s][k] != 0.f) atomicAdd(g + size_t(s) * NH * 4 + k, dwr[s][k]);
+                for (int k = 0; k < 4; ++k)
+                    if (dwr[s][k] != 0.f) atomicAdd(d + k, dwr[s][k]);
+            }
+        }
+    }
     }
 }
 
@@ -829,6 +841,8 @@ int wbp_geometry(const pc_code* c, int64_t B, size_t real_bytes, bool backward, 
     if (fixed + slot > size_t(optin)) return PC_EUNSUPPORTED;
     int slots = int((size_t(optin) - fixed) / slot);
     slots = std::max(1, std::min({slots, 15, (reg ? 512 : 1024) / g->tps}));
+    // a batch that does not fill the chip goes to more SMs with fewer frames each
+    slots = int(std::max<int64_t>(1, std::min<int64_t>(slots, (B + sms - 1) / sms)));
     g->slots = slots;
     g->smem = fixed + size_t(slots) * slot;
     g->grid = int(std::min<int64_t>(int64_t(sms), (B + slots - 1) / slots));
@@ -921,13 +935,13 @@ int forward_impl(const pc_code* c, const Real* llr, const Real* w, int32_t T, in
     P->T = T;
     P->tps = g.tps;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(ws, 0, 8, st) != cudaSuccess) return PC_ECUDA;
     if constexpr (std::is_same<Real, float>::value) {
         // FP32 from N = 16 to 1024 (the unrolled backward reads its checkpoints in the sw32
         // layout; at N = 8 that layout is the natural order the generic kernel writes)
         if (c->n >= 4 && c->n <= 10)
             return launch_forward_reg(c->n, *P, g, st) == cudaSuccess ? PC_OK : PC_ECUDA;
     }
+    if (cudaMemsetAsync(ws, 0, 8, st) != cudaSuccess) return PC_ECUDA;
     if (cudaFuncSetAttribute(wbp_forward_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) !=
         cudaSuccess)
         return PC_ECUDA;
@@ -966,8 +980,15 @@ int backward_impl(const pc_code* c, const Real* llr, const Real* w, int32_t T, i
     state[0] = reinterpret_cast<Real*>(static_cast<unsigned char*>(ws) + 256);
     state[1] = state[0] + size_t(B) * size_t(c->n - 1) * size_t(c->N);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if constexpr (std::is_same<Real, float>::value) {
+        if (reg) {
+            // one launch; the kernel takes the two gradient states in turn, from the first on
+            P->gin = P->gout = state[0];
+            return launch_backward_reg(c->n, *P, g, st) == cudaSuccess ? PC_OK : PC_ECUDA;
+        }
+    }
     if (gllr && cudaMemsetAsync(gllr, 0, size_t(B) * c->N * sizeof(Real), st) != cudaSuccess) return PC_ECUDA;
-    if (!reg && cudaFuncSetAttribute(wbp_backward_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(wbp_backward_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       int(g.smem)) != cudaSuccess)
         return PC_ECUDA;
     for (int it = T - 1; it >= 0; --it) {
@@ -975,12 +996,6 @@ int backward_impl(const pc_code* c, const Real* llr, const Real* w, int32_t T, i
         P->gin = state[(T - 1 - it) & 1];      // written by the launch of iteration it+1 (unused at it = T-1)
         P->gout = state[(T - it) & 1];
         if (cudaMemsetAsync(ws, 0, 8, st) != cudaSuccess) return PC_ECUDA;
-        if constexpr (std::is_same<Real, float>::value) {
-            if (reg) {
-                if (launch_backward_reg(c->n, *P, g, st) != cudaSuccess) return PC_ECUDA;
-                continue;
-            }
-        }
         wbp_backward_kernel<Real><<<g.grid, g.slots * g.tps, g.smem, st>>>(*P);
         if (cudaGetLastError() != cudaSuccess) return PC_ECUDA;
     }
