@@ -238,6 +238,9 @@ Kernel kernel_for(int n, int N, int tpf, int fk)
     const char* v = std::getenv("PCBP_DECODER");
     if (v && std::strcmp(v, "grouped") == 0) return kGrouped;
     if (n >= 7 && v && std::strcmp(v, "tmem") == 0) return kTmem;
+#ifdef PCBP_CHECKED
+    if (n >= 7) return kTmem;      // the kernel with the range checks
+#endif
     return warp_kernel_has(n, fk) ? kWarp : kTmem;
 }
 
@@ -341,6 +344,9 @@ int plan_launch4(const pc_code* c, int64_t B, int fk, LaunchGeom* g, int slots_r
     slots = int(std::max<int64_t>(1, std::min<int64_t>(slots, (B + di.sms - 1) / di.sms)));
     int max_slots = 0;
     shape4_of(c->n, c->K, slots, &max_slots, &smem);
+    // over half of an SM's shared memory: two CTAs with tensor-memory allocations never share an SM,
+    // and the allocation never waits
+    smem = std::max(smem, size_t(di.smem_per_sm) / 2 + 1024);
     if (smem > size_t(di.smem_optin)) return PC_EUNSUPPORTED;
     g->slots = slots;
     g->smem = smem;
