@@ -212,15 +212,6 @@ void shape4_of(int n, int K, int slots, int* max_slots, size_t* smem)
 #undef PCBP_SHAPE4
 }
 
-int occupancy4_of(int n, const LaunchGeom& g, int fk)
-{
-    int occ = 0;
-#define PCBP_OCC4(k) occ = bp4_occupancy_##k(g, fk)
-    PCBP_SWITCH_N(n, PCBP_OCC4)
-#undef PCBP_OCC4
-    return occ;
-}
-
 cudaError_t launch4_of(int n, const WarpParams& P, const LaunchGeom& g, int fk, cudaStream_t st, bool pdl)
 {
     cudaError_t e = cudaSuccess;
@@ -332,7 +323,7 @@ int plan_launch3(const pc_code* c, int64_t B, int fk, LaunchGeom* g, int slots_r
 // Register-resident kernel: as many frames per CTA as it is built for; where the batch does not
 // fill the chip, fewer frames per CTA on more SMs (a frame alone on its SM takes about half the
 // time per iteration of one that shares it).
-int plan_launch4(const pc_code* c, int64_t B, int fk, LaunchGeom* g, int slots_req = 0)
+int plan_launch4(const pc_code* c, int64_t B, LaunchGeom* g, int slots_req = 0)
 {
     DeviceInfo di;
     int rc = device_info(&di);
@@ -344,16 +335,12 @@ int plan_launch4(const pc_code* c, int64_t B, int fk, LaunchGeom* g, int slots_r
     slots = int(std::max<int64_t>(1, std::min<int64_t>(slots, (B + di.sms - 1) / di.sms)));
     int max_slots = 0;
     shape4_of(c->n, c->K, slots, &max_slots, &smem);
-    // over half of an SM's shared memory: two CTAs with tensor-memory allocations never share an SM,
-    // and the allocation never waits
+    // over half of an SM's shared memory: one CTA per SM, so the tensor-memory allocation never waits
     smem = std::max(smem, size_t(di.smem_per_sm) / 2 + 1024);
     if (smem > size_t(di.smem_optin)) return PC_EUNSUPPORTED;
     g->slots = slots;
     g->smem = smem;
-    g->grid = 1;
-    const int occ = occupancy4_of(c->n, *g, fk);
-    if (occ < 1) return PC_EUNSUPPORTED;
-    g->grid = int(std::min<int64_t>((B + slots - 1) / slots, int64_t(di.sms) * occ));
+    g->grid = int(std::min<int64_t>((B + slots - 1) / slots, di.sms));
     return PC_OK;
 }
 
@@ -447,11 +434,14 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
     if (!trace && kind == kWarp) {
         std::unique_ptr<WarpParams> W(new WarpParams);
         fill_warp_params(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, W.get());
-        rc = plan_launch4(code, B, sched->fkind, &g);
+        rc = plan_launch4(code, B, &g);
         if (rc != PC_OK) return rc;
         W->slots = g.slots;
-        W->counter = reinterpret_cast<unsigned long long*>(d_workspace);
-        if (cudaMemsetAsync(d_workspace, 0, 32, st) != cudaSuccess) return PC_ECUDA;
+        // a batch with a slot for every frame needs no counter (and its memset no place in the stream)
+        if (B > int64_t(g.grid) * g.slots) {
+            W->counter = reinterpret_cast<unsigned long long*>(d_workspace);
+            if (cudaMemsetAsync(d_workspace, 0, 32, st) != cudaSuccess) return PC_ECUDA;
+        }
         return launch4_of(code->n, *W, g, sched->fkind, st, false) == cudaSuccess ? PC_OK : PC_ECUDA;
     }
     std::unique_ptr<BpParams> P(new BpParams);
@@ -653,7 +643,7 @@ extern "C" int bp_mixed_prepare(const pc_batch* batches, int32_t n_batches, void
         if (b.B > 0) {
             const Kernel kind = kernel_for(b.code->n, b.code->N, b.threads_per_frame, b.sched.fkind);
             m->kernel = kind;
-            const int rc = kind == kWarp   ? plan_launch4(b.code, b.B, b.sched.fkind, &m->g, b.slots)
+            const int rc = kind == kWarp   ? plan_launch4(b.code, b.B, &m->g, b.slots)
                  : kind == kTmem ? plan_launch3(b.code, b.B, b.sched.fkind, &m->g, b.slots)
                                  : plan_launch2(b.code, b.B, b.sched.fkind, &m->g, b.slots);
             if (rc != PC_OK) return rc;
@@ -707,7 +697,7 @@ extern "C" int bp_slot_limit(const pc_code* code, int32_t threads_per_frame, int
         return PC_EUNSUPPORTED;
     LaunchGeom g;
     const Kernel kind = kernel_for(code->n, N, tpf, fkind);
-    rc = kind == kWarp   ? plan_launch4(code, INT32_MAX, fkind, &g)
+    rc = kind == kWarp   ? plan_launch4(code, INT32_MAX, &g)
          : kind == kTmem ? plan_launch3(code, 1, fkind, &g)
                          : plan_launch2(code, 1, fkind, &g);
     if (rc != PC_OK) return rc;

@@ -35,30 +35,12 @@ cudaError_t launch_variant(const WarpParams& P, const LaunchGeom& g, cudaStream_
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, P);
 }
-
-template <int FK>
-int occupancy(const LaunchGeom& g)
-{
-    auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, 0>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) != cudaSuccess)
-        return 0;
-    int blocks = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, g.slots * 32 * Geo::WPF, g.smem) != cudaSuccess)
-        return 0;
-    return blocks;
-}
 }  // namespace
 
 void PCBP_CAT(bp4_shape_, PCBP_LOGN)(int K, int slots, int* max_slots_out, size_t* smem_out)
 {
     *max_slots_out = Geo::SLOTS;
     *smem_out = Geo::smem_bytes(K, slots);
-}
-
-int PCBP_CAT(bp4_occupancy_, PCBP_LOGN)(const LaunchGeom& g, int fkind)
-{
-    if (fkind) return warp_kernel_has(PCBP_LOGN, 1) ? occupancy<PCBP_LOGN <= 6 ? 1 : 0>(g) : 0;
-    return occupancy<0>(g);
 }
 
 cudaError_t PCBP_CAT(bp4_launch_, PCBP_LOGN)(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st,

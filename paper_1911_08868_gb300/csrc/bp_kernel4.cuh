@@ -722,8 +722,9 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
         // The index is drawn only now: drawn a frame ahead, a frame waits for the long one (up to
         // max_iters) that its warp is at.  N = 256 2.5 dB, 12,800 frames 775 -> 535 us; 50,021 frames at
         // 3 dB 576 -> 472 us; N = 1024 9.18 -> 8.99 ms on 262,144, N = 2048 7.72 -> 7.34 ms on 16,384.
+        // Without a counter every frame has its own slot, and total is past the last.
         Index nf = 0;
-        if (lane == 0 && warp == 0) nf = Index(atomicAdd(P.counter, 1ull));
+        if (P.counter && lane == 0 && warp == 0) nf = Index(atomicAdd(P.counter, 1ull));
         __syncwarp();
         if constexpr (WPF > 1) {
             if (tid == 0) *reinterpret_cast<Index*>(red + 8) = nf;

@@ -65,7 +65,6 @@ struct WarpParams;
 
 #define PCBP_DECLARE_LEN4(n)                                                                       \
     void bp4_shape_##n(int K, int slots, int* max_slots_out, size_t* smem_out);                    \
-    int bp4_occupancy_##n(const LaunchGeom& g, int fkind);                                         \
     cudaError_t bp4_launch_##n(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st, bool pdl);
 
 PCBP_DECLARE_LEN4(3)

@@ -57,3 +57,25 @@ def test_register_kernel_equals_grouped_kernel(pcbp, monkeypatch, N, sched):
                 out.append([t.cpu().numpy() for t in dec(llr)])
             for a, b in zip(*out):
                 assert np.array_equal(a, b), (K, r, B)
+
+
+@pytest.mark.parametrize("N,slots", [(64, 24), (256, 16), (512, 8), (2048, 2)])
+def test_batches_around_one_frame_per_slot(pcbp, monkeypatch, N, slots):
+    """A batch with a slot for every frame runs without a frame counter (whatever the workspace
+    holds), one frame more with it."""
+    import torch
+
+    dev = gpu_device()
+    full = slots * torch.cuda.get_device_properties(dev).multi_processor_count
+    code = pcbp.pc_construct(N, N // 2, 8, 0x9B)
+    gen = torch.Generator(device=dev).manual_seed(N)
+    llr = torch.randn((full + 1, N), generator=gen, device=dev) * 3.0 + 2.0
+    s = pcbp.sched(mode=0, stop_kind=1, stop_from=1)
+    monkeypatch.setenv("PCBP_DECODER", "grouped")
+    want = [t.cpu().numpy() for t in pcbp.Decoder(code, s, 8, dev)(llr)]
+    monkeypatch.setenv("PCBP_DECODER", "")
+    for B in (full - 1, full, full + 1):
+        dec = pcbp.Decoder(code, s, 8, dev)
+        dec.workspace.fill_(0x5A)
+        for a, b in zip(dec(llr[:B]), want):
+            assert np.array_equal(a.cpu().numpy(), b[:B]), B
