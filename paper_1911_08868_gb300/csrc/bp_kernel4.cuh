@@ -320,13 +320,24 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
     // --- exchanges through the scratch plane
     // natural labels, layout a -> layout b: a warp writes the positions that it read last, so no
     // barrier is needed before
-    auto exch = [&](auto ga, auto gb, float* v) {
+    auto exch = [&](auto evc, auto ga, auto gb, float* v) {
         constexpr int a = decltype(ga)::value, b = decltype(gb)::value;
-        __syncwarp();
-        plane_st<LOGN, a>(scratch, tb[a], v);
-        if constexpr (Geo::top_warps(a) && Geo::top_warps(b)) __syncwarp();
-        else fsync();
-        plane_ld<LOGN, b>(scratch, tb[b], v);
+        if constexpr (KB == 1 && n >= 5 && !decltype(evc)::value) {
+            // neighbouring layouts swap the register bit with one lane bit: a shuffle (60,000 frames of
+            // N = 64 for 100 iterations 1,295 -> 814 us, N = 32 716 -> 680; no gain at N = 8 and 16, and
+            // none under an event, where the boundary also has the other exchange)
+            constexpr int bit = 1 << (n - 2 - (a < b ? a : b));
+            const bool up = (lane & bit) != 0;
+            const float y = __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], bit);
+            v[0] = up ? y : v[0];
+            v[1] = up ? v[1] : y;
+        } else {
+            __syncwarp();
+            plane_st<LOGN, a>(scratch, tb[a], v);
+            if constexpr (Geo::top_warps(a) && Geo::top_warps(b)) __syncwarp();
+            else fsync();
+            plane_ld<LOGN, b>(scratch, tb[b], v);
+        }
     };
     // a level at the places of a map (byte distances from the scratch plane)
     auto map_ld = [&](const float* plane, const int* map, float* v) {
@@ -389,13 +400,13 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
         constexpr int g = decltype(gc)::value, b = Geo::first(g + 1);
         std::integral_constant<int, g + 1> gn;
         if (decltype(evc)::value && ev_hi == b - 1) exch_out(lead(std::integral_constant<int, b>{}), map_hi, gn, v);
-        else exch(gc, gn, v);
+        else exch(evc, gc, gn, v);
     };
     // and of the R sweep, from group g to g - 1
     auto r_boundary = [&](auto evc, auto gc, float* v) {
         constexpr int g = decltype(gc)::value, b = Geo::first(g);
         if (decltype(evc)::value && ev_hi == b - 1) exch_in(gc, map_hi, v);
-        else exch(gc, std::integral_constant<int, g - 1>{}, v);
+        else exch(evc, gc, std::integral_constant<int, g - 1>{}, v);
     };
     // R(n+1) in the layout and labels of stage n-1
     auto priors = [&](auto evc, float* v) {
