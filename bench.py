@@ -96,7 +96,7 @@ def kernel_sha() -> str:
     import re
 
     h = hashlib.sha256()
-    for name in ("bp_kernel.cuh", "bp_kernel2.cuh", "bp_kernel3.cuh", "bp_inst3.cu"):
+    for name in ("bp_kernel.cuh", "bp_kernel2.cuh", "bp_kernel3.cuh", "bp_kernel4.cuh", "bp_inst4.cu"):
         text = (ROOT / "paper_1911_08868_gb300" / "csrc" / name).read_text()
         text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
         text = re.sub(r"//[^\n]*", "", text)
@@ -113,7 +113,7 @@ def profiled_traffic(sha: str):
     """DRAM bytes per launch of FRAMES frames from the committed ncu summary, if it was taken on this
     kernel source (the caller scales it to the launch's frame count: the traffic is one LLR read and
     one result write per frame)."""
-    p = ROOT / "profiles" / "bp_decode_tmem_n1024_pp_s4t10.md"
+    p = ROOT / "profiles" / "bp_decode_warp_n1024_pp_s4t10.md"
     if not p.exists():
         return None
     vals = {}

@@ -179,7 +179,7 @@ int bp_decode_trace(const pc_code* code, const float* d_llr, const pc_sched* sch
                     int32_t* d_iters, uint8_t* d_crc_ok, void* d_workspace,
                     void* stream);
 
-/* bp_decode (Algorithm 1) through the same production kernel, which also
+/* bp_decode (Algorithm 1) through the tensor-memory kernel, which also
  * records the messages at both ends of the factor graph after each frame's
  * last iteration, for verification of the message arithmetic (Sec. II-B)
  * where the outputs alone would hide it (the exact box-plus f).
@@ -188,7 +188,7 @@ int bp_decode_trace(const pc_code* code, const float* d_llr, const pc_sched* sch
  *     level 1 (the channel side), both after frame b's last iteration, whose
  *     R sweep is always completed.  Left untouched when max_iters is 0.
  *   Other arguments and outputs as bp_decode (the outputs are equal).
- * Returns PC_EUNSUPPORTED for N < 128 (those lengths run another kernel) or
+ * Returns PC_EUNSUPPORTED for N < 128 (that kernel starts at N = 128) or
  * with the G-matrix stop test (stop_kind & 2). */
 int bp_decode_posterior(const pc_code* code, const float* d_llr, const pc_sched* sched,
                         int32_t max_iters, int64_t B, uint32_t* d_bits, int32_t* d_iters,
@@ -232,8 +232,8 @@ int wbp_forward(const pc_code* code, const float* d_llr, const float* d_w, int32
                 float* d_logits, float* d_ckpt, void* d_workspace, void* stream);
 /* Given d_glogits = dLoss/dlogits [B][K]: d_gw += dLoss/dw (caller zeroes it
  * for a fresh gradient); d_gllr (nullable) = dLoss/dllr [B][N].  Runs the
- * iterations in reverse, each recomputed from its checkpoint: in one launch for
- * N <= 1024, else (and in FP64) in one launch per iteration. */
+ * iterations in reverse, each recomputed from its checkpoint: in FP32 up to
+ * N = 1024 in one launch where that is faster, else one launch per iteration. */
 int wbp_backward(const pc_code* code, const float* d_llr, const float* d_w, int32_t T, int64_t B,
                  const float* d_ckpt, const float* d_glogits, float* d_gw, float* d_gllr,
                  void* d_workspace, void* stream);
@@ -273,7 +273,7 @@ typedef struct {
     int32_t slots;            /* frames resident per CTA; 0 = as many as fit */
     int32_t threads_per_frame;/* 0: the bp_decode kernel for this N; otherwise the count of one of
                                  the other two kernels as bp_kernel_threads reports it (TMEM-resident stage
-                                 groups: N/4 for N = 128..512, N/8 for 1024 and 2048;
+                                 groups: N/4 up to N = 256, N/8 from N = 512;
                                  shared-memory groups: max(32, N/4)); anything else is
                                  PC_EUNSUPPORTED */
     int32_t reserved;         /* 0 */

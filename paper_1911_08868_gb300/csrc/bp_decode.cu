@@ -583,7 +583,7 @@ extern "C" int bp_decode_host(const pc_code* code, const float* h_llr, const pc_
 namespace pcbp {
 namespace {
 
-constexpr uint32_t kMixedMagic = 0x70636278u;
+constexpr uint32_t kMixedMagic = 0x70636279u;   // changes with the layout of MixedEntry
 
 struct MixedEntry {
     union {

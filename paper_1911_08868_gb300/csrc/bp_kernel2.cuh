@@ -1,6 +1,6 @@
 // Stage-grouped PP-BP decoder kernel for sm_103a (Algorithm 1 of arXiv
-// 1911.08868): the bp_decode path for N < 128 (and for every N when
-// PCBP_DECODER=grouped); its stage partition and swizzled planes are also the
+// 1911.08868): bp_decode with PCBP_DECODER=grouped, and batches of a mixed
+// sweep that ask for its threads per frame; its stage partition and swizzled planes are also the
 // base of the TMEM kernel (bp_kernel3.cuh).
 //
 // Same arithmetic as bp_kernel.cuh (every FP32 operation explicitly rounded,

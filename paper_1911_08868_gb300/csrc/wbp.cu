@@ -5,7 +5,7 @@
 // 3 R_out2) in place of the fixed min-sum scale.  Forward keeps the R planes
 // at every iteration boundary as checkpoints; backward runs the iterations in
 // reverse, recomputes each from its checkpoint and applies the adjoint of the
-// R sweep then of the L sweep (FP32 up to N = 1024 in one launch, else one
+// R sweep then of the L sweep (FP32 up to N = 1024 in one launch where that is faster, else one
 // launch per iteration).
 //
 // Derivatives of f_w(a, b) = w sign(a) sign(b) min(|a|, |b|): with a the
@@ -561,10 +561,9 @@ __global__ void __launch_bounds__(1024, 1) wbp_backward_kernel(const __grid_cons
 // at levels 1..n+1, two gradient planes between R levels and G, the incoming gradient (levels
 // 2..n): (5n+2) N floats, in the sw32 layout.  Between two stages of butterfly distance at most
 // 32 a warp waits only for itself (stage_sync); the gradient planes are left zero by the stage
-// that consumes them, so a frame starts without clearing them; the next frame's index and this
-// frame's accumulated LLR gradient are read early and used later, so neither round trip stalls
-// the slot.
-template <int LOGN>
+// that consumes them, so a frame starts without clearing them; the frame's accumulated LLR
+// gradient is read early and added later, so its round trip does not stall the slot.
+template <int LOGN, bool ALL>
 __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_constant__ WbpParams<float> P)
 {
     constexpr int n = LOGN, N = 1 << LOGN, NH = N / 2;
@@ -594,11 +593,12 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
     const int slots = blockDim.x / tps;
     const bool act = tid < NH;                 // N < 64: fewer elements than a warp
     const int q = act ? tid : 0;
-    // One launch runs the iterations in reverse, with a fixed share of the frames in each slot (the
-    // gradient of R(t) that a frame leaves is read again by the same slot only): no launch, counter
-    // and drain between iterations.  Forth and back over the frames, so that an iteration starts with
-    // the gradients written last, which L2 still holds.
-    for (int it = P.T - 1; it >= 0; --it) {
+    // One launch runs the iterations in reverse (ALL) or one of them, with a fixed share of the frames in
+    // each slot (the gradient of R(t) that a frame leaves is read again by the same slot only): no
+    // counter, and with ALL no launch and drain between iterations.  Forth and back over the frames, so
+    // that an iteration starts with the gradients written last, which L2 still holds (N = 1024, T = 10
+    // 2,023 against 2,054 us).
+    for (int it = ALL ? P.T - 1 : P.it; it >= (ALL ? 0 : P.it); --it) {
     const bool last = it == P.T - 1;
     float dwr[n][4];
 #pragma unroll
@@ -620,8 +620,8 @@ __global__ void __launch_bounds__(512, 1) wbp_backward_reg_kernel(const __grid_c
     for (int f = back ? f0 + fs * (left - 1) : f0; left > 0; --left, f += f_step) {
         // the buffers' addresses from a copy of `it` the compiler cannot see through: held across the
         // frames they would take six of the 128 registers (backward 5% slower at N = 1024)
-        int iv = it;
-        asm volatile("" : "+r"(iv));
+        int iv = ALL ? it : P.it;
+        if (ALL) asm volatile("" : "+r"(iv));
         wt = P.w + size_t(iv) * n * NH * 4;
         float* gout = P.gout + (size_t((P.T - iv) & 1) * P.B + size_t(f)) * (n - 1) * N;
         // inputs of the frame: the checkpoint R(it), the LLRs (L level 1) and (before the last
@@ -886,29 +886,45 @@ cudaError_t launch_forward_reg(int n, const WbpParams<float>& P, const Geo& g, c
 #undef PCBP_WBP_FWD
 }
 
-// The register-accumulating FP32 backward, instantiated for n = 3..10.
+// The register-accumulating FP32 backward, instantiated for n = 3..10, all iterations in one launch
+// or one launch for each.
+template <int LOGN, bool ALL>
+cudaError_t launch_backward_reg_of(const WbpParams<float>& P, const Geo& g, cudaStream_t st)
+{
+    auto kern = wbp_backward_reg_kernel<LOGN, ALL>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    if (e != cudaSuccess) return e;
+    if (ALL) {
+        kern<<<g.grid, g.slots * g.tps, g.smem, st>>>(P);
+        return cudaGetLastError();
+    }
+    std::unique_ptr<WbpParams<float>> Q(new WbpParams<float>(P));
+    for (int it = P.T - 1; it >= 0 && e == cudaSuccess; --it) {
+        Q->it = it;
+        kern<<<g.grid, g.slots * g.tps, g.smem, st>>>(*Q);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
 cudaError_t launch_backward_reg(int n, const WbpParams<float>& P, const Geo& g, cudaStream_t st)
 {
-#define PCBP_WBP_REG(k)                                                                                      \
-    case k: {                                                                                                \
-        cudaError_t e = cudaFuncSetAttribute(wbp_backward_reg_kernel<k>,                                     \
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));      \
-        if (e != cudaSuccess) return e;                                                                      \
-        wbp_backward_reg_kernel<k><<<g.grid, g.slots * g.tps, g.smem, st>>>(P);                              \
-        return cudaGetLastError();                                                                           \
-    }
     switch (n) {
-        PCBP_WBP_REG(3)
-        PCBP_WBP_REG(4)
-        PCBP_WBP_REG(5)
-        PCBP_WBP_REG(6)
-        PCBP_WBP_REG(7)
-        PCBP_WBP_REG(8)
-        PCBP_WBP_REG(9)
-        PCBP_WBP_REG(10)
+        case 3: return launch_backward_reg_of<3, true>(P, g, st);
+        case 4: return launch_backward_reg_of<4, true>(P, g, st);
+        case 5: return launch_backward_reg_of<5, true>(P, g, st);
+        case 6: return launch_backward_reg_of<6, true>(P, g, st);
+        case 7: return launch_backward_reg_of<7, true>(P, g, st);
+        case 8: return launch_backward_reg_of<8, true>(P, g, st);
+        case 9: return launch_backward_reg_of<9, true>(P, g, st);
+        case 10:
+            // With the iteration a launch parameter a frame costs 4% less (two registers of the 128), a
+            // launch about 5 us: T = 20 at batch 4,096 3,756 against 3,916 us, T = 10 2,023 / 2,090, at
+            // batch 2,048 (13 frames a slot) 2,020 / 2,026, at 300 448 / 346, T = 5 at 1,000 308 / 288.
+            return P.B >= 12 * int64_t(g.grid) * g.slots ? launch_backward_reg_of<10, false>(P, g, st)
+                                                         : launch_backward_reg_of<10, true>(P, g, st);
         default: return cudaErrorInvalidValue;
     }
-#undef PCBP_WBP_REG
 }
 
 template <typename Real>
@@ -982,7 +998,7 @@ int backward_impl(const pc_code* c, const Real* llr, const Real* w, int32_t T, i
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if constexpr (std::is_same<Real, float>::value) {
         if (reg) {
-            // one launch; the kernel takes the two gradient states in turn, from the first on
+            // the kernel takes the two gradient states in turn, from the first on
             P->gin = P->gout = state[0];
             return launch_backward_reg(c->n, *P, g, st) == cudaSuccess ? PC_OK : PC_ECUDA;
         }

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("T", [1, 2, 5])
-@pytest.mark.parametrize("N,B", [(16, 1), (16, 333), (128, 5), (128, 2100), (256, 700), (1024, 3), (1024, 310)])
+@pytest.mark.parametrize("N,B", [(16, 1), (16, 333), (128, 5), (128, 2100), (256, 700), (1024, 3), (1024, 310), (1024, 2100)])
 def test_batch_is_the_sum_of_its_frames(pcbp, N, B, T):
     import torch
 
