@@ -39,7 +39,7 @@
 // Time per frame-iteration against the tensor-memory kernel: without an event 0.38 / 0.94 ns at
 // N = 256, 0.86 / 1.36 at 512, 2.17 / 3.47 at 1024, 5.09 / 7.48 at 2048; under an event 0.50 / 1.17,
 // 1.19 / 1.50, 3.10 / 3.75 and 7.36 / 8.75; a switch 1.2 / 2.1, 2.7 / 6.9, 6.3 / 7.1 and 15.5 / 16.
-// N = 64 (100,003 PP-BP frames at 3 dB) 1.13 ms against 5.97 ms of the shared-memory kernel.
+// N = 64 (100,003 PP-BP frames at 3 dB) 0.95 ms against 5.95 ms of the shared-memory kernel.
 //
 // Arithmetic: every floating-point operation and its operand order are those of the other decoder
 // kernels (l_layer, r_layer), so the outputs are bit-identical.
