@@ -3,6 +3,7 @@
 // translation units compile in parallel.
 #include "bp_kernel.cuh"
 #include "bp_launch.h"
+#include "launch_smem.h"
 
 #ifndef PCBP_LOGN
 #error "PCBP_LOGN must be defined"
@@ -18,8 +19,8 @@ template <bool TRACE, int FK>
 cudaError_t launch_variant(const BpParams& P, const LaunchGeom& g, cudaStream_t st)
 {
     constexpr int T = threads_per_slot<PCBP_LOGN>();
-    auto kern = bp_decode_kernel<PCBP_LOGN, T, TRACE, FK>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    constexpr auto kern = bp_decode_kernel<PCBP_LOGN, T, TRACE, FK>;
+    const cudaError_t e = allow_dynamic_smem<kern>();
     if (e != cudaSuccess) return e;
     kern<<<g.grid, g.slots * T, g.smem, st>>>(P);
     return cudaGetLastError();
@@ -29,9 +30,8 @@ template <bool TRACE, int FK>
 int occupancy(const LaunchGeom& g)
 {
     constexpr int T = threads_per_slot<PCBP_LOGN>();
-    auto kern = bp_decode_kernel<PCBP_LOGN, T, TRACE, FK>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) != cudaSuccess)
-        return 0;
+    constexpr auto kern = bp_decode_kernel<PCBP_LOGN, T, TRACE, FK>;
+    if (allow_dynamic_smem<kern>() != cudaSuccess) return 0;
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, g.slots * T, g.smem) != cudaSuccess) return 0;
     return blocks;

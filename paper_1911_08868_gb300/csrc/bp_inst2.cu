@@ -2,6 +2,7 @@
 // 2^PCBP_LOGN (compiled once per n = 3..11).
 #include "bp_kernel2.cuh"
 #include "bp_launch.h"
+#include "launch_smem.h"
 
 #ifndef PCBP_LOGN
 #error "PCBP_LOGN must be defined"
@@ -25,8 +26,8 @@ using Geo = G2<PCBP_LOGN, KBSEL>;
 template <int FK>
 cudaError_t launch_variant(const BpParams& P, const LaunchGeom& g, cudaStream_t st, bool pdl)
 {
-    auto kern = bp_decode_grouped_kernel<PCBP_LOGN, KBSEL, FK>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    constexpr auto kern = bp_decode_grouped_kernel<PCBP_LOGN, KBSEL, FK>;
+    const cudaError_t e = allow_dynamic_smem<kern>();
     if (e != cudaSuccess) return e;
     if (!pdl) {
         kern<<<g.grid, g.slots * Geo::T, g.smem, st>>>(P);
@@ -48,9 +49,8 @@ cudaError_t launch_variant(const BpParams& P, const LaunchGeom& g, cudaStream_t 
 template <int FK>
 int occupancy(const LaunchGeom& g)
 {
-    auto kern = bp_decode_grouped_kernel<PCBP_LOGN, KBSEL, FK>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) != cudaSuccess)
-        return 0;
+    constexpr auto kern = bp_decode_grouped_kernel<PCBP_LOGN, KBSEL, FK>;
+    if (allow_dynamic_smem<kern>() != cudaSuccess) return 0;
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, g.slots * Geo::T, g.smem) != cudaSuccess)
         return 0;

@@ -3,6 +3,7 @@
 // 2^KB positions, KB = tmem_default_kb(n) unless PCBP_KB3 sets it).
 #include "bp_kernel3.cuh"
 #include "bp_launch.h"
+#include "launch_smem.h"
 
 #ifndef PCBP_LOGN
 #error "PCBP_LOGN must be defined"
@@ -25,8 +26,8 @@ using Geo = G3<PCBP_LOGN, KB>;
 template <int FK, int WG, int PO = 0>
 cudaError_t launch_variant(const BpParams& P, const LaunchGeom& g, cudaStream_t st, bool pdl)
 {
-    auto kern = bp_decode_tmem_kernel<PCBP_LOGN, KB, FK, WG, PO>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    constexpr auto kern = bp_decode_tmem_kernel<PCBP_LOGN, KB, FK, WG, PO>;
+    const cudaError_t e = allow_dynamic_smem<kern>();
     if (e != cudaSuccess) return e;
     if (!pdl) {
         kern<<<g.grid, g.slots * Geo::T, g.smem, st>>>(P);
@@ -48,9 +49,8 @@ cudaError_t launch_variant(const BpParams& P, const LaunchGeom& g, cudaStream_t 
 template <int FK>
 int occupancy(const LaunchGeom& g)
 {
-    auto kern = bp_decode_tmem_kernel<PCBP_LOGN, KB, FK, 0, 0>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) != cudaSuccess)
-        return 0;
+    constexpr auto kern = bp_decode_tmem_kernel<PCBP_LOGN, KB, FK, 0, 0>;
+    if (allow_dynamic_smem<kern>() != cudaSuccess) return 0;
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, g.slots * Geo::T, g.smem) != cudaSuccess)
         return 0;

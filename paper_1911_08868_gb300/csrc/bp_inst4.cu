@@ -2,6 +2,7 @@
 // 2^PCBP_LOGN (compiled once per n = 3..11).
 #include "bp_kernel4.cuh"
 #include "bp_launch.h"
+#include "launch_smem.h"
 
 #ifndef PCBP_LOGN
 #error "PCBP_LOGN must be defined"
@@ -20,8 +21,8 @@ using Geo = G4<PCBP_LOGN>;
 template <int FK, int WG>
 cudaError_t launch_variant(const WarpParams& P, const LaunchGeom& g, cudaStream_t st, bool pdl)
 {
-    auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, WG>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    constexpr auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, WG>;
+    const cudaError_t e = allow_dynamic_smem<kern>();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(g.grid));

@@ -244,10 +244,8 @@ template <int LOGN>
 int launch_encode(const EncParams& P, int sms, cudaStream_t st)
 {
     using Geo = EncGeo<LOGN>;
+    static_assert(Geo::smem(Geo::N) <= 48 * 1024, "within the default limit of dynamic shared memory");
     const size_t smem = Geo::smem(P.K);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(encode_kernel<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-        return PC_ECUDA;
     // persistent CTAs (the table is made once per CTA; 4, 6 and 8 per SM measured alike)
     const int64_t tiles = (P.B + Geo::WARPS * Geo::FPW - 1) / (Geo::WARPS * Geo::FPW);
     const int grid = int(std::min<int64_t>(tiles, int64_t(sms) * kEncodeCtas));

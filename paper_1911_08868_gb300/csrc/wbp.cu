@@ -21,6 +21,7 @@
 #include <memory>
 #include <type_traits>
 
+#include "launch_smem.h"
 #include "pcbp_internal.h"
 
 namespace pcbp {
@@ -867,8 +868,7 @@ cudaError_t launch_forward_reg(int n, const WbpParams<float>& P, const Geo& g, c
 {
 #define PCBP_WBP_FWD(k)                                                                                      \
     case k: {                                                                                                \
-        cudaError_t e = cudaFuncSetAttribute(wbp_forward_reg_kernel<k>,                                      \
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));      \
+        const cudaError_t e = allow_dynamic_smem<wbp_forward_reg_kernel<k>>();                               \
         if (e != cudaSuccess) return e;                                                                      \
         wbp_forward_reg_kernel<k><<<g.grid, g.slots * g.tps, g.smem, st>>>(P);                               \
         return cudaGetLastError();                                                                           \
@@ -891,8 +891,8 @@ cudaError_t launch_forward_reg(int n, const WbpParams<float>& P, const Geo& g, c
 template <int LOGN, bool ALL>
 cudaError_t launch_backward_reg_of(const WbpParams<float>& P, const Geo& g, cudaStream_t st)
 {
-    auto kern = wbp_backward_reg_kernel<LOGN, ALL>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem));
+    constexpr auto kern = wbp_backward_reg_kernel<LOGN, ALL>;
+    cudaError_t e = allow_dynamic_smem<kern>();
     if (e != cudaSuccess) return e;
     if (ALL) {
         kern<<<g.grid, g.slots * g.tps, g.smem, st>>>(P);
@@ -958,9 +958,7 @@ int forward_impl(const pc_code* c, const Real* llr, const Real* w, int32_t T, in
             return launch_forward_reg(c->n, *P, g, st) == cudaSuccess ? PC_OK : PC_ECUDA;
     }
     if (cudaMemsetAsync(ws, 0, 8, st) != cudaSuccess) return PC_ECUDA;
-    if (cudaFuncSetAttribute(wbp_forward_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(g.smem)) !=
-        cudaSuccess)
-        return PC_ECUDA;
+    if (allow_dynamic_smem<wbp_forward_kernel<Real>>() != cudaSuccess) return PC_ECUDA;
     wbp_forward_kernel<Real><<<g.grid, g.slots * g.tps, g.smem, st>>>(*P);
     return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ECUDA;
 }
@@ -1004,9 +1002,7 @@ int backward_impl(const pc_code* c, const Real* llr, const Real* w, int32_t T, i
         }
     }
     if (gllr && cudaMemsetAsync(gllr, 0, size_t(B) * c->N * sizeof(Real), st) != cudaSuccess) return PC_ECUDA;
-    if (cudaFuncSetAttribute(wbp_backward_kernel<Real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      int(g.smem)) != cudaSuccess)
-        return PC_ECUDA;
+    if (allow_dynamic_smem<wbp_backward_kernel<Real>>() != cudaSuccess) return PC_ECUDA;
     for (int it = T - 1; it >= 0; --it) {
         P->it = it;
         P->gin = state[(T - 1 - it) & 1];      // written by the launch of iteration it+1 (unused at it = T-1)
