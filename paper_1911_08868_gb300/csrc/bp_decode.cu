@@ -12,26 +12,6 @@
 
 namespace pcbp {
 
-int device_info(DeviceInfo* out)
-{
-    static DeviceInfo cache[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PC_ECUDA;
-    if (dev < 64 && cache[dev].sms > 0) {
-        *out = cache[dev];
-        return PC_OK;
-    }
-    DeviceInfo d;
-    if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return PC_ECUDA;
-    if (cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
-        return PC_ECUDA;
-    if (cudaDeviceGetAttribute(&d.smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
-        return PC_ECUDA;
-    if (dev < 64) cache[dev] = d;
-    *out = d;
-    return PC_OK;
-}
-
 namespace {
 
 void shape_of(int n, int* T, size_t* slot)

@@ -1,8 +1,12 @@
 // Host side of libpcbp: code construction, argument validation and the
 // tables the kernels read.
+#include <cuda_runtime.h>
+
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -40,6 +44,35 @@ static std::vector<uint32_t> xpow_table(int count, int r, uint64_t g)
         if ((v >> r) & 1ull) v ^= g;
     }
     return pw;
+}
+
+int device_info(DeviceInfo* out)
+{
+    // filled by the first call on each device, which may run in several threads at once
+    static DeviceInfo cache[64];
+    static std::atomic<bool> filled[64];
+    static std::mutex filling;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return PC_ECUDA;
+    if (dev < 64 && filled[dev].load(std::memory_order_acquire)) {
+        *out = cache[dev];
+        return PC_OK;
+    }
+    DeviceInfo d;
+    if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return PC_ECUDA;
+    if (cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return PC_ECUDA;
+    if (cudaDeviceGetAttribute(&d.smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
+        return PC_ECUDA;
+    if (dev < 64) {
+        std::lock_guard<std::mutex> lock(filling);
+        if (!filled[dev].load(std::memory_order_relaxed)) {
+            cache[dev] = d;
+            filled[dev].store(true, std::memory_order_release);
+        }
+    }
+    *out = d;
+    return PC_OK;
 }
 
 int validate_code(const pc_code* c)

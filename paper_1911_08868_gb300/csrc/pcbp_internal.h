@@ -97,7 +97,7 @@ struct EncParams {
     int64_t B;
 };
 
-// The current device (bp_decode.cu).
+// The current device (pcbp_host.cpp).
 struct DeviceInfo {
     int sms = 0;
     int smem_optin = 0;
