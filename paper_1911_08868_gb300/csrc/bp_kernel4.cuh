@@ -664,6 +664,9 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                     } else {
                         const int2 w = *reinterpret_cast<const int2*>(d);
                         ao[2 * q] = w.x; ao[2 * q + 1] = w.y;
+                        // below N = 64 two or more lanes stand for one thread: all of them read the old map
+                        // before one writes the new
+                        if constexpr (T < 32) __syncwarp();
                         *reinterpret_cast<int2*>(d) = make_int2(aw[2 * q], aw[2 * q + 1]);
                     }
                 }
