@@ -418,10 +418,14 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
         if (rc != PC_OK) return rc;
         W->slots = g.slots;
         // a batch with a slot for every frame needs no counter (and its memset no place in the stream)
-        if (B > int64_t(g.grid) * g.slots) {
-            W->counter = reinterpret_cast<unsigned long long*>(d_workspace);
-            if (cudaMemsetAsync(d_workspace, 0, 32, st) != cudaSuccess) return PC_ECUDA;
-        }
+        const bool counted = B > int64_t(g.grid) * g.slots;
+        if (counted) W->counter = reinterpret_cast<unsigned long long*>(d_workspace);
+#ifdef PCBP_CHECKED
+        const size_t clear = 32;       // the counter and the status word, whether they are used or not
+#else
+        const size_t clear = counted ? 32 : 0;
+#endif
+        if (clear && cudaMemsetAsync(d_workspace, 0, clear, st) != cudaSuccess) return PC_ECUDA;
         return launch4_of(code->n, *W, g, sched->fkind, st, false) == cudaSuccess ? PC_OK : PC_ECUDA;
     }
     std::unique_ptr<BpParams> P(new BpParams);
