@@ -209,9 +209,6 @@ Kernel kernel_for(int n, int N, int tpf, int fk)
     const char* v = std::getenv("PCBP_DECODER");
     if (v && std::strcmp(v, "grouped") == 0) return kGrouped;
     if (n >= 7 && v && std::strcmp(v, "tmem") == 0) return kTmem;
-#ifdef PCBP_CHECKED
-    if (n >= 7) return kTmem;      // the kernel with the range checks
-#endif
     return warp_kernel_has(n, fk) ? kWarp : kTmem;
 }
 
@@ -421,7 +418,8 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
         const bool counted = B > int64_t(g.grid) * g.slots;
         if (counted) W->counter = reinterpret_cast<unsigned long long*>(d_workspace);
 #ifdef PCBP_CHECKED
-        const size_t clear = 32;       // the counter and the status word, whether they are used or not
+        const size_t clear = 32;       // the counter and the status word at byte 16, whether they are used or not
+        W->job.check = reinterpret_cast<unsigned*>(static_cast<unsigned char*>(d_workspace) + 16);
 #else
         const size_t clear = counted ? 32 : 0;
 #endif

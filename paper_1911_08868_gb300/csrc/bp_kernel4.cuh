@@ -166,44 +166,61 @@ __device__ __forceinline__ void sfor(F&& f)
     }
 }
 
+// Index i of `step` consecutive entries, a multiple of step, in a buffer of `limit`.  A build with
+// PCBP_CHECKED checks it: out of range, bit `cls` of the status word (when there is one) is set and
+// the access redirected to entry 0, so nothing faults.
+template <int step = 1>
+__device__ __forceinline__ int in_range(unsigned* status, unsigned cls, int i, int limit)
+{
+#ifdef PCBP_CHECKED
+    if (i < 0 || i > limit - step || i % step != 0) {
+        chk_fail(status, cls);
+        return 0;
+    }
+#endif
+    return i;
+}
+
 // A level between a thread's registers and a plane, in the layout of group g: tb is the word of
 // the thread's base position, the registers are at compile-time distances from it.
 template <int LOGN, int g>
-__device__ __forceinline__ void plane_st(float* plane, int tb, const float* v)
+__device__ __forceinline__ void plane_st(float* plane, int tb, const float* v, unsigned* check)
 {
     using Geo = G4<LOGN>;
     constexpr int E = Geo::E;
     if constexpr (g == Geo::G - 1) {
 #pragma unroll
         for (int e = 0; e < E; e += Geo::VT) {
-            if constexpr (E >= 4) *reinterpret_cast<float4*>(plane + tb + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-            else *reinterpret_cast<float2*>(plane + tb + e) = make_float2(v[e], v[e + 1]);
+            float* const d = plane + in_range<Geo::VT>(check, 0, tb + e, Geo::PLANE);
+            if constexpr (E >= 4) *reinterpret_cast<float4*>(d) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+            else *reinterpret_cast<float2*>(d) = make_float2(v[e], v[e + 1]);
         }
     } else {
 #pragma unroll
-        for (int e = 0; e < E; ++e) plane[tb + Geo::word_of(Geo::epos(g, e))] = v[e];
+        for (int e = 0; e < E; ++e) plane[in_range(check, 0, tb + Geo::word_of(Geo::epos(g, e)), Geo::PLANE)] = v[e];
     }
 }
 
 template <int LOGN, int g>
-__device__ __forceinline__ void plane_ld(const float* plane, int tb, float* v)
+__device__ __forceinline__ void plane_ld(const float* plane, int tb, float* v, unsigned* check)
 {
     using Geo = G4<LOGN>;
     constexpr int E = Geo::E;
     if constexpr (g == Geo::G - 1) {
 #pragma unroll
         for (int e = 0; e < E; e += Geo::VT) {
+            const float* const s = plane + in_range<Geo::VT>(check, 0, tb + e, Geo::PLANE);
             if constexpr (E >= 4) {
-                const float4 w = *reinterpret_cast<const float4*>(plane + tb + e);
+                const float4 w = *reinterpret_cast<const float4*>(s);
                 v[e] = w.x; v[e + 1] = w.y; v[e + 2] = w.z; v[e + 3] = w.w;
             } else {
-                const float2 w = *reinterpret_cast<const float2*>(plane + tb + e);
+                const float2 w = *reinterpret_cast<const float2*>(s);
                 v[e] = w.x; v[e + 1] = w.y;
             }
         }
     } else {
 #pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = plane[tb + Geo::word_of(Geo::epos(g, e))];
+        for (int e = 0; e < E; ++e) v[e] = plane[in_range(check, 0, tb + Geo::word_of(Geo::epos(g, e)), Geo::PLANE)];
     }
 }
 
@@ -333,27 +350,32 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
             v[1] = up ? v[1] : y;
         } else {
             __syncwarp();
-            plane_st<LOGN, a>(scratch, tb[a], v);
+            plane_st<LOGN, a>(scratch, tb[a], v, J.check);
             if constexpr (Geo::top_warps(a) && Geo::top_warps(b)) __syncwarp();
             else fsync();
-            plane_ld<LOGN, b>(scratch, tb[b], v);
+            plane_ld<LOGN, b>(scratch, tb[b], v, J.check);
         }
     };
-    // a level at the places of a map (byte distances from the scratch plane)
+    // a level at the places of a map (byte distances from the start of a plane)
+    auto map_at = [&](const int* map, int i) {
+        const int from = int(map - maps);
+        return map + (in_range<VT>(J.check, 3, from + i, G * N) - from);
+    };
+    auto place = [&](int d) { return in_range<4>(J.check, 3, d, 4 * Geo::PLANE); };
     auto map_ld = [&](const float* plane, const int* map, float* v) {
         const char* p = reinterpret_cast<const char*>(plane);
 #pragma unroll
         for (int q = 0; q < E / VT; ++q) {
             if constexpr (VT == 4) {
-                const int4 w = *reinterpret_cast<const int4*>(map + (q * T + tid) * 4);
-                v[4 * q] = *reinterpret_cast<const float*>(p + w.x);
-                v[4 * q + 1] = *reinterpret_cast<const float*>(p + w.y);
-                v[4 * q + 2] = *reinterpret_cast<const float*>(p + w.z);
-                v[4 * q + 3] = *reinterpret_cast<const float*>(p + w.w);
+                const int4 w = *reinterpret_cast<const int4*>(map_at(map, (q * T + tid) * 4));
+                v[4 * q] = *reinterpret_cast<const float*>(p + place(w.x));
+                v[4 * q + 1] = *reinterpret_cast<const float*>(p + place(w.y));
+                v[4 * q + 2] = *reinterpret_cast<const float*>(p + place(w.z));
+                v[4 * q + 3] = *reinterpret_cast<const float*>(p + place(w.w));
             } else {
-                const int2 w = *reinterpret_cast<const int2*>(map + (q * T + tid) * 2);
-                v[2 * q] = *reinterpret_cast<const float*>(p + w.x);
-                v[2 * q + 1] = *reinterpret_cast<const float*>(p + w.y);
+                const int2 w = *reinterpret_cast<const int2*>(map_at(map, (q * T + tid) * 2));
+                v[2 * q] = *reinterpret_cast<const float*>(p + place(w.x));
+                v[2 * q + 1] = *reinterpret_cast<const float*>(p + place(w.y));
             }
         }
     };
@@ -362,15 +384,15 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
 #pragma unroll
         for (int q = 0; q < E / VT; ++q) {
             if constexpr (VT == 4) {
-                const int4 w = *reinterpret_cast<const int4*>(map + (q * T + tid) * 4);
-                *reinterpret_cast<float*>(p + w.x) = v[4 * q];
-                *reinterpret_cast<float*>(p + w.y) = v[4 * q + 1];
-                *reinterpret_cast<float*>(p + w.z) = v[4 * q + 2];
-                *reinterpret_cast<float*>(p + w.w) = v[4 * q + 3];
+                const int4 w = *reinterpret_cast<const int4*>(map_at(map, (q * T + tid) * 4));
+                *reinterpret_cast<float*>(p + place(w.x)) = v[4 * q];
+                *reinterpret_cast<float*>(p + place(w.y)) = v[4 * q + 1];
+                *reinterpret_cast<float*>(p + place(w.z)) = v[4 * q + 2];
+                *reinterpret_cast<float*>(p + place(w.w)) = v[4 * q + 3];
             } else {
-                const int2 w = *reinterpret_cast<const int2*>(map + (q * T + tid) * 2);
-                *reinterpret_cast<float*>(p + w.x) = v[2 * q];
-                *reinterpret_cast<float*>(p + w.y) = v[2 * q + 1];
+                const int2 w = *reinterpret_cast<const int2*>(map_at(map, (q * T + tid) * 2));
+                *reinterpret_cast<float*>(p + place(w.x)) = v[2 * q];
+                *reinterpret_cast<float*>(p + place(w.y)) = v[2 * q + 1];
             }
         }
     };
@@ -382,12 +404,12 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
         else __syncwarp();
         map_st(map, v);
         fsync();
-        plane_ld<LOGN, b>(ev_plane, tb[b], v);
+        plane_ld<LOGN, b>(ev_plane, tb[b], v, J.check);
     };
     auto exch_in = [&](auto ga, const int* map, float* v) {
         constexpr int a = decltype(ga)::value;
         __syncwarp();
-        plane_st<LOGN, a>(ev_plane, tb[a], v);
+        plane_st<LOGN, a>(ev_plane, tb[a], v, J.check);
         fsync();
         map_ld(ev_plane, map, v);
     };
@@ -411,7 +433,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
     // R(n+1) in the layout and labels of stage n-1
     auto priors = [&](auto evc, float* v) {
         if (decltype(evc)::value && ev_hi == n - 1) map_ld(s_pri, map_hi, v);
-        else plane_ld<LOGN, G - 1>(s_pri, tb[G - 1], v);
+        else plane_ld<LOGN, G - 1>(s_pri, tb[G - 1], v, J.check);
     };
     // --- frame queue: the first frames spread over the SMs, the others from the counter
     // (a batch of 2^31 frames of N >= 512 would hold over 4 TB of LLRs)
@@ -420,9 +442,15 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
     const Index total = Index(gridDim.x) * P.slots;
     Index f = Index(slot) * Index(gridDim.x) + Index(blockIdx.x);
     auto load_llr = [&](Index fi) {
+#ifdef PCBP_CHECKED
+        if (fi < 0 || fi >= frames) {
+            chk_fail(J.check, 5);
+            fi = 0;
+        }
+#endif
         const float* src = J.llr + size_t(fi) * N + tid;     // the first group's thread bits are the low bits
 #pragma unroll
-        for (int e = 0; e < E; ++e) Lc[e] = __ldg(src + Geo::epos(0, e));
+        for (int e = 0; e < E; ++e) Lc[e] = __ldg(src + (in_range(J.check, 5, tid + Geo::epos(0, e), N) - tid));
     };
     if (f < frames) load_llr(f);
 
@@ -494,7 +522,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                 constexpr int CB = Geo::CB;
 #pragma unroll
                 for (int k = 0; k < E / CB; ++k)
-                    res ^= s_crc[((k << CB) + int((um >> (CB * k)) & ((1u << CB) - 1u))) * T + tid];
+                    res ^= s_crc[in_range(J.check, 2, ((k << CB) + int((um >> (CB * k)) & ((1u << CB) - 1u))) * T + tid, Geo::CRC_WORDS)];
                 if (T < 32 && lane >= T) res = 0;
                 res = __reduce_xor_sync(0xffffffffu, res);
                 if constexpr (WPF > 1) {
@@ -556,7 +584,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                 for (int e = 0; e < E; ++e) {
                     const unsigned b = __ballot_sync(0xffffffffu, x[e] < 0.f);
                     if constexpr (n >= 6) {
-                        if (lane == 0) xh[(Geo::epos(0, e) >> 5) | warp] = b;
+                        if (lane == 0) xh[in_range(J.check, 2, (Geo::epos(0, e) >> 5) | warp, Geo::NW)] = b;
                     } else {
                         w0 |= (b & ((1u << (T & 31)) - 1u)) << Geo::epos(0, e);
                     }
@@ -565,7 +593,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                 unsigned v = um << ((tid << KB) & 31);
 #pragma unroll
                 for (int o = 1; o < 32 / E && o < T; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
-                dec[(tid << KB) >> 5] = v;
+                dec[in_range(J.check, 2, (tid << KB) >> 5, Geo::NW)] = v;
                 fsync();
                 const bool gok = g_check<LOGN>(dec, xh, lane);
                 fsync();
@@ -656,7 +684,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                 }
 #pragma unroll
                 for (int q = 0; q < E / VT; ++q) {
-                    int* d = mp + (q * T + tid) * VT;
+                    int* d = mp + (in_range<VT>(J.check, 3, g * N + (q * T + tid) * VT, G * N) - g * N);
                     if constexpr (VT == 4) {
                         const int4 w = *reinterpret_cast<const int4*>(d);
                         ao[4 * q] = w.x; ao[4 * q + 1] = w.y; ao[4 * q + 2] = w.z; ao[4 * q + 3] = w.w;
@@ -679,7 +707,8 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                     const bool move_old = k <= ev_hi && !zero_old, move_new = k <= hi && !zero_new;
                     const unsigned z_old = zero_old ? in_old : 0u, z_new = zero_new ? in_new : 0u;
                     float v[E];
-                    slot_ld<E>(tm + uint32_t(k * E), v);
+                    const uint32_t col = tm + uint32_t(in_range<E>(J.check, 1, k * E, Geo::SLOT_COLS));
+                    slot_ld<E>(col, v);
                     tm_wait_ld();
                     tm_fence<E>(v);
                     char* const pl = reinterpret_cast<char*>(ev_plane);
@@ -689,18 +718,18 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                         fsync();
                         if (move_old) {
 #pragma unroll
-                            for (int e = 0; e < E; ++e) *reinterpret_cast<float*>(pl + ao[e]) = v[e];
+                            for (int e = 0; e < E; ++e) *reinterpret_cast<float*>(pl + place(ao[e])) = v[e];
                         } else {
 #pragma unroll
-                            for (int e = 0; e < E; ++e) *reinterpret_cast<float*>(pl + an[e]) = v[e];
+                            for (int e = 0; e < E; ++e) *reinterpret_cast<float*>(pl + place(an[e])) = v[e];
                         }
                         fsync();
 #pragma unroll
-                        for (int e = 0; e < E; ++e) v[e] = *reinterpret_cast<const float*>(pl + (move_new ? aw[e] : an[e]));
+                        for (int e = 0; e < E; ++e) v[e] = *reinterpret_cast<const float*>(pl + place(move_new ? aw[e] : an[e]));
                     }
 #pragma unroll
                     for (int e = 0; e < E; ++e) v[e] = (z_new >> e) & 1u ? 0.f : v[e];
-                    slot_st<E>(tm + uint32_t(k * E), v);
+                    slot_st<E>(col, v);
                 }
             }
             tm_wait_st();
@@ -713,7 +742,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
             // the channel LLRs under the new labels
             load_llr(f);
             fsync();
-            plane_st<LOGN, 0>(ev_plane, tb[0], Lc);
+            plane_st<LOGN, 0>(ev_plane, tb[0], Lc, J.check);
             fsync();
             map_ld(ev_plane, maps, Lc);
             fsync();
@@ -747,7 +776,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
             unsigned v = um << ((tid << KB) & 31);
 #pragma unroll
             for (int o = 1; o < 32 / E && o < T; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
-            dec[(tid << KB) >> 5] = v;
+            dec[in_range(J.check, 2, (tid << KB) >> 5, Geo::NW)] = v;
         }
         fsync();
         if constexpr (WPF > 1) nf = *reinterpret_cast<const Index*>(red + 8);
@@ -760,14 +789,14 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
             const int kk = o * 32 + lane;
             uint32_t bit = 0;
             if (kk < K) {
-                const int pos = s_info[kk];
+                const int pos = in_range(J.check, 2, s_info[kk], N);
                 bit = (dec[pos >> 5] >> (pos & 31)) & 1u;
             }
             const uint32_t word = __ballot_sync(0xffffffffu, bit);
             if (lane == ((o / WPF) & 31)) w = word;
             if (((o / WPF) & 31) == 31 || o + WPF >= KW) {
                 const int oo = o - ((o / WPF) & 31) * WPF + lane * WPF;
-                if (oo <= o) J.bits[size_t(fo) * KW + oo] = w;
+                if (oo <= o) J.bits[size_t(fo) * KW + in_range(J.check, 4, oo, KW)] = w;
             }
         }
         if (lane == 0 && warp == 0) {
