@@ -201,6 +201,15 @@ cudaError_t launch4_of(int n, const WarpParams& P, const LaunchGeom& g, int fk, 
     return e;
 }
 
+cudaError_t launch4_post_of(int n, const WarpParams& P, const LaunchGeom& g, cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+#define PCBP_LAUNCH4(k) e = bp4_launch_post_##k(P, g, st)
+    PCBP_SWITCH_N(n, PCBP_LAUNCH4)
+#undef PCBP_LAUNCH4
+    return e;
+}
+
 // The kernel of a batch that asks for tpf threads per frame (0: the decoder's choice, the
 // register-resident kernel where it is built).
 Kernel kernel_for(int n, int N, int tpf, int fk)
@@ -379,8 +388,9 @@ void fill_warp_params(const pc_code* code, const float* d_llr, const pc_sched* s
     build_warp_code(code, P);
 }
 
-// d_post (posterior output, nullable): the TMEM kernel's debug build that also writes L at node
-// level n+1 and R at node level 1 of every frame's last iteration.
+// d_post (messages output, nullable): the variant of the same kernel that also writes L at node
+// level n+1 and R at node level 1 of every frame's last iteration (the shared-memory kernel has
+// none: the TMEM kernel in its place).
 int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched, int32_t max_iters, int64_t B,
                   bool trace, const pc_event* h_events, int32_t n_events, float* d_dump, uint32_t* d_bits,
                   int32_t* d_iters, uint8_t* d_crc_ok, void* d_workspace, void* stream, float* d_post = nullptr)
@@ -407,7 +417,8 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
     }
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     LaunchGeom g;
-    const Kernel kind = d_post ? kTmem : kernel_for(code->n, code->N, 0, sched->fkind);
+    Kernel kind = kernel_for(code->n, code->N, 0, sched->fkind);
+    if (d_post && kind == kGrouped) kind = kTmem;
     if (!trace && kind == kWarp) {
         std::unique_ptr<WarpParams> W(new WarpParams);
         fill_warp_params(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, W.get());
@@ -424,7 +435,10 @@ int decode_common(const pc_code* code, const float* d_llr, const pc_sched* sched
         const size_t clear = counted ? 32 : 0;
 #endif
         if (clear && cudaMemsetAsync(d_workspace, 0, clear, st) != cudaSuccess) return PC_ECUDA;
-        return launch4_of(code->n, *W, g, sched->fkind, st, false) == cudaSuccess ? PC_OK : PC_ECUDA;
+        W->job.post = d_post;
+        const cudaError_t e = d_post ? launch4_post_of(code->n, *W, g, st)
+                                     : launch4_of(code->n, *W, g, sched->fkind, st, false);
+        return e == cudaSuccess ? PC_OK : PC_ECUDA;
     }
     std::unique_ptr<BpParams> P(new BpParams);
     fill_params(code, d_llr, sched, max_iters, B, d_bits, d_iters, d_crc_ok, P.get());

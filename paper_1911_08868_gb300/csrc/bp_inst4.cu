@@ -18,10 +18,10 @@ using Geo = G4<PCBP_LOGN>;
 
 // pdl: programmatic dependent launch, the grid may start while the previous
 // kernel of the stream still runs (for independent batches).
-template <int FK, int WG>
+template <int FK, int WG, int PO = 0>
 cudaError_t launch_variant(const WarpParams& P, const LaunchGeom& g, cudaStream_t st, bool pdl)
 {
-    constexpr auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, WG>;
+    constexpr auto kern = bp_decode_warp_kernel<PCBP_LOGN, FK, WG, PO>;
     const cudaError_t e = allow_dynamic_smem<kern>();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -54,6 +54,17 @@ cudaError_t PCBP_CAT(bp4_launch_, PCBP_LOGN)(const WarpParams& P, const LaunchGe
         return wg ? launch_variant<FK, 1>(P, g, st, pdl) : launch_variant<FK, 0>(P, g, st, pdl);
     }
     return wg ? launch_variant<0, 1>(P, g, st, pdl) : launch_variant<0, 0>(P, g, st, pdl);
+}
+
+// Scaled min-sum with the messages output (CRC stop or none; P.job.post set).
+cudaError_t PCBP_CAT(bp4_launch_post_, PCBP_LOGN)(const WarpParams& P, const LaunchGeom& g, cudaStream_t st)
+{
+#if PCBP_LOGN >= 7
+    if ((P.job.S.stop_kind & 2) || P.job.S.fkind) return cudaErrorInvalidValue;
+    return launch_variant<0, 0, 1>(P, g, st, false);
+#else
+    return cudaErrorInvalidValue;
+#endif
 }
 
 }  // namespace pcbp

@@ -274,7 +274,9 @@ static __device__ __noinline__ void draw_events(const DevSched& S, int n, uint64
                           int(uint32_t(ord >> 32)));
 }
 
-template <int LOGN, int FK, int WG>
+// PO = 1 (the messages output of bp_decode_posterior, for verification): a frame's last iteration
+// completes its R sweep and writes L at node level n+1 and R at node level 1 to J.post.
+template <int LOGN, int FK, int WG, int PO>
 __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, uint32_t tm_base)
 {
     using Geo = G4<LOGN>;
@@ -288,6 +290,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
     const float alpha = S.alpha, nz = J.neg_zero;
     const int max_iters = J.max_iters;
     constexpr bool want_g = WG != 0;
+    static_assert(!(PO && (WG || LOGN < 7)), "the messages output is built for the CRC stop, from N = 128 on");
     const bool want_crc = (S.stop_kind & 1) != 0;
 
     const float* s_pri = smem;                                             // priors, a plane
@@ -470,6 +473,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
         auto iterate = [&](auto evc) -> bool {
             constexpr bool EV = decltype(evc)::value;
             float x[E], pr[E];
+            float lu[PO ? E : 1];                  // PO: L(n+1), natural labels
             // ---------------- L sweep
 #pragma unroll
             for (int e = 0; e < E; ++e) x[e] = Lc[e];
@@ -506,6 +510,10 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
             bool gtest = false;
             if (check || it == max_iters) {
                 if (EV && ev_hi == n - 1) exch_out(std::false_type{}, map_hi, std::integral_constant<int, G - 1>{}, x);
+                if constexpr (PO != 0) {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) lu[e] = x[e];
+                }
                 // the sign of x + 0 is set exactly where x < 0 (-0 becomes +0)
                 um = 0;
 #pragma unroll
@@ -571,8 +579,22 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
                 }
             };
             r_group(std::integral_constant<int, 0>{});
-            if (last_iteration()) return true;
+            const bool last = last_iteration();
+            if (!PO && last) return true;
             sfor<1, G>(r_group);
+            if constexpr (PO != 0) {
+                if (last) {
+                    r_layer<E, FK>(x, Lc, Geo::stage_reg(0), alpha, nz);
+                    if constexpr (EV) exch_out(std::true_type{}, maps, std::integral_constant<int, 0>{}, x);
+                    float* const post = J.post + size_t(f) * 2 * N;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        post[(tid << KB) + e] = lu[e];
+                        post[N + tid + Geo::epos(0, e)] = x[e];
+                    }
+                    return true;
+                }
+            }
             // ---------------- G-matrix test: u G_N against the hard decisions of L1 + R1
             if (want_g && gtest) {
                 r_layer<E, FK>(x, Lc, Geo::stage_reg(0), alpha, nz);
@@ -807,7 +829,7 @@ __device__ __forceinline__ void warp_frames(const WarpParams& P, float* smem, ui
     }
 }
 
-template <int LOGN, int FK, int WG>
+template <int LOGN, int FK, int WG, int PO = 0>
 __global__ void __launch_bounds__(32 * G4<LOGN>::WARPS, 1)
     bp_decode_warp_kernel(const __grid_constant__ WarpParams P)
 {
@@ -853,7 +875,7 @@ __global__ void __launch_bounds__(32 * G4<LOGN>::WARPS, 1)
         s_crc[i] = c;
     }
     __syncthreads();
-    if (int(threadIdx.x) < P.slots * 32 * Geo::WPF) warp_frames<LOGN, FK, WG>(P, smem4, tm_base);
+    if (int(threadIdx.x) < P.slots * 32 * Geo::WPF) warp_frames<LOGN, FK, WG, PO>(P, smem4, tm_base);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

@@ -65,7 +65,8 @@ struct WarpParams;
 
 #define PCBP_DECLARE_LEN4(n)                                                                       \
     void bp4_shape_##n(int K, int slots, int* max_slots_out, size_t* smem_out);                    \
-    cudaError_t bp4_launch_##n(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st, bool pdl);
+    cudaError_t bp4_launch_##n(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st, bool pdl); \
+    cudaError_t bp4_launch_post_##n(const WarpParams& P, const LaunchGeom& g, cudaStream_t st);
 
 PCBP_DECLARE_LEN4(3)
 PCBP_DECLARE_LEN4(4)
