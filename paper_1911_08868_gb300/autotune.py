@@ -8,7 +8,8 @@ Threads per frame: 0 (the kernel bp_decode runs) and the counts bp_kernel_thread
 reports for the two others (TMEM-resident stage groups: N/4 up to N = 256, N/8 from
 512; shared-memory groups: max(32, N/4); where they coincide the library runs the
 TMEM kernel).  Results are cached per GPU
-name, library build and schedule in a JSON file ($PCBP_TUNE_CACHE, default ~/.cache/pcbp_tune.json).
+name, library build, kernel choice (PCBP_DECODER) and schedule in a JSON file ($PCBP_TUNE_CACHE, default
+~/.cache/pcbp_tune.json).
 """
 from __future__ import annotations
 
@@ -62,7 +63,9 @@ def tune_launch(lengths, sched_for, max_iters: int = 300, frames: int = 16384, e
     dev = torch.device(device)
     lib = pcbp.library_path()
     # a rebuilt library (new kernels) is tuned afresh
-    key = f"{torch.cuda.get_device_name(dev)}|{lib}|{os.stat(lib).st_mtime_ns}|{max_iters}|{frames}|{ebn0}|capped"
+    # PCBP_DECODER: what threads per frame 0 (and a count that two kernels share) selects
+    key = (f"{torch.cuda.get_device_name(dev)}|{lib}|{os.stat(lib).st_mtime_ns}|{max_iters}|{frames}|{ebn0}|capped|"
+           f"{os.environ.get('PCBP_DECODER', '')}")
     cache = {}
     cp = cache_path()
     if use_cache and cp.exists():
