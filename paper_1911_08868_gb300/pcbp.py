@@ -170,7 +170,11 @@ def _stream(stream):
     if stream is None:
         import torch
 
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # torch's own call for it saves a microsecond of a 16 us call; it is not part of torch's interface
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return torch.cuda.current_stream().cuda_stream
+        return raw(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
