@@ -136,15 +136,18 @@ int bp_decode_workspace_size(const pc_code* code, int64_t B, size_t* bytes);
  * keeps each stage group's interior messages in tensor memory (groups of 2
  * stages up to N = 256, of 3 from 512).  The environment variable PCBP_DECODER
  * selects the latter for every f (tmem, N >= 128) or the shared-memory
- * stage-grouped kernel (grouped); the outputs are the same.  The frames of a call share a persistent grid: each CTA holds one
- * frame per slot and fetches the next frame index from d_workspace. */
+ * stage-grouped kernel (grouped); the outputs are the same.  The frames of a
+ * call share a persistent grid: each CTA holds one frame per slot, and a slot
+ * that ends its frame takes the next index from a counter in d_workspace (the
+ * register-resident kernel leaves d_workspace alone where the batch fits the
+ * slots). */
 int bp_decode(const pc_code* code, const float* d_llr, const pc_sched* sched,
               int32_t max_iters, int64_t B, uint32_t* d_bits, int32_t* d_iters,
               uint8_t* d_crc_ok, void* d_workspace, void* stream);
 
 /* bp_decode (Algorithm 1) on buffers that stay in host memory: the decoder
- * reads each frame's LLRs once and writes its results in place across the
- * host-device link (NVLink-C2C on Grace-Blackwell systems), with no staging
+ * reads each frame's LLRs as the frame starts (and again at each of its
+ * switches) and writes its results in place across the host-device link (NVLink-C2C on Grace-Blackwell systems), with no staging
  * copies.  The paper has no counterpart; the operation is bp_decode's.
  *   h_llr, h_bits, h_iters, h_crc_ok: laid out as d_llr, d_bits, d_iters,
  *     d_crc_ok of bp_decode (h_llr 16-byte aligned), each in page-locked

@@ -1,5 +1,8 @@
 // Instantiates the stage-grouped decoder kernel for one code length,
-// 2^PCBP_LOGN (compiled once per n = 3..11).
+// 2^PCBP_LOGN (compiled once per n = 3..11).  No call runs it unless asked to
+// (PCBP_DECODER=grouped, a batch's threads per frame): it is kept as the
+// reference that the other decoder kernels are compared with, bit for bit, at
+// sizes the oracle cannot reach.
 #include "bp_kernel2.cuh"
 #include "bp_launch.h"
 #include "launch_smem.h"

@@ -1,6 +1,9 @@
 // Instantiates the TMEM-resident stage-grouped decoder kernel for one code
 // length, 2^PCBP_LOGN (compiled once per n = 7..11: every lane of a warp owns
-// 2^KB positions, KB = tmem_default_kb(n) unless PCBP_KB3 sets it).
+// 2^KB positions, KB = tmem_default_kb(n) unless PCBP_KB3 sets it).  Exact
+// box-plus is what calls run of it; its scaled min-sum (PCBP_DECODER=tmem, a
+// batch's threads per frame) is kept as a second reference for the
+// register-resident kernel, messages included.
 #include "bp_kernel3.cuh"
 #include "bp_launch.h"
 #include "launch_smem.h"

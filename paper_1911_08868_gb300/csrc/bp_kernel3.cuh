@@ -1,8 +1,7 @@
 // Stage-grouped PP-BP decoder kernel with group-private messages in tensor
 // memory (sm_103a TMEM), the bp_decode path for exact box-plus at N >= 128
-// (Algorithm 1 of arXiv 1911.08868); scaled min-sum runs it for the posterior
-// output, with PCBP_DECODER=tmem, and where a mixed sweep asks for its threads
-// per frame.
+// (Algorithm 1 of arXiv 1911.08868); scaled min-sum runs it with
+// PCBP_DECODER=tmem and where a mixed sweep asks for its threads per frame.
 //
 // Positions per thread, swizzled shared-memory planes, stop tests and switch
 // follow the stage-grouped kernel (bp_kernel2.cuh), and so does every

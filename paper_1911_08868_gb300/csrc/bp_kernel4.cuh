@@ -36,10 +36,12 @@
 // test comes after the R sweep's last group, which hides the reduction and the warps' skew (N = 1024
 // at 3 dB 10.0 -> 9.7 ms on 262,144 frames, N = 2048 at 2 dB 8.2 -> 7.7 ms on 16,384).
 //
-// Time per frame-iteration against the tensor-memory kernel: without an event 0.38 / 0.94 ns at
-// N = 256, 0.86 / 1.36 at 512, 2.17 / 3.47 at 1024, 5.09 / 7.48 at 2048; under an event 0.50 / 1.17,
-// 1.19 / 1.50, 3.10 / 3.75 and 7.36 / 8.75; a switch 1.2 / 2.1, 2.7 / 6.9, 6.3 / 7.1 and 15.5 / 16.
-// N = 64 (100,003 PP-BP frames at 3 dB) 0.95 ms against 5.95 ms of the shared-memory kernel.
+// Time per frame-iteration against the tensor-memory kernel (14,592 frames of scaled min-sum without
+// a stop test, 100 iterations more against 100 fewer; events of 4 stages), in ns, at N = 128, 256, 512,
+// 1024 and 2048: without an event 0.27 / 0.51, 0.39 / 0.95, 0.88 / 1.39, 2.22 / 3.59 and 5.20 / 7.62;
+// under an event 0.36 / 0.55, 0.55 / 1.24, 1.23 / 1.62, 3.20 / 3.85 and 7.47 / 8.87; a switch 0.86 / 1.69,
+// 1.27 / 2.97, 2.89 / 4.63, 6.83 / 7.59 and 16.2 / 16.5.  N = 64 against the shared-memory kernel: 0.13 /
+// 0.89, 0.24 / 1.14 and 0.80 / 3.04.
 //
 // Arithmetic: every floating-point operation and its operand order are those of the other decoder
 // kernels (l_layer, r_layer), so the outputs are bit-identical.
@@ -67,7 +69,12 @@ struct G4 {
     static constexpr int P = 36;
     static constexpr int PLANE = N >= 32 ? (N / 32) * P : N;
 
-    // first stage of group g: groups of KB stages (N = 1024: 3, 3, 2, 2)
+    // First stage of group g: groups of KB stages.  N = 1024 has 3, 3, 2, 2: with 3, 3, 3, 1 the third
+    // group's register bits would be position bits 1..3, and a warp's accesses in that layout would
+    // meet in pairs on the banks (position bits 0, 4, 5, .. from the lanes); from run_low = 2 on they
+    // do not.  Without an event 2.22 against 2.35 ns per frame-iteration, 262,144 PP-BP frames at 3 dB
+    // 8.97 against 9.35 ms, 65,536 at 2 dB 14.1 against 14.7.  No other length leaves one stage but
+    // N = 128, whose groups are of 2.
     __host__ __device__ static constexpr int first(int g) { return g >= G ? n : (n == 10 && g == 3 ? 8 : g * KB); }
     __host__ __device__ static constexpr int len(int g) { return first(g + 1) - first(g); }
     __host__ __device__ static constexpr int grp(int s) { return n == 10 && s == 8 ? 3 : s / KB; }
@@ -125,8 +132,11 @@ struct G4 {
     // whether the iteration under an event has a copy of each group's stages with the tests for a
     // relabelling inside the group, entered where it relabels there: fewer instructions (a test
     // makes the values of both paths meet in the same registers, with moves), more code.  Pays at
-    // N = 1024 (9.07 against 9.68 ms on 262,144 PP-BP frames at 3 dB); N = 512 2.75 against 2.56 ms
-    // (32,768 frames, CRC and G-matrix stop), N = 2048 8.00 against 7.71 (16,384 frames at 2 dB).
+    // N = 1024 alone.  PP-BP frames, with the copies against without: N = 1024 8.97 / 9.50 ms (262,144 at
+    // 3 dB) and 3.48 / 3.72 (65,536, CRC and G-matrix stop); N = 128 0.87 / 0.85 (100,003); N = 256
+    // 0.73 / 0.71 and 1.08 / 1.02, N = 512 1.64 / 1.51 and 2.31 / 2.15 (65,536, CRC stop and both);
+    // N = 2048 7.62 / 7.50 (16,384 at 2 dB) and 2.81 / 2.83 (32,768 at 3 dB).  Below N = 128 every group
+    // is one stage, and there is nothing to copy.
     static constexpr bool COPY = n == 10;
     // tensor memory: n-1 slots of E columns per warp, WARPS / 4 warps to a lane quarter
     static constexpr int SLOT_COLS = (n - 1) * E;

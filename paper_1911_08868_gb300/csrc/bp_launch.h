@@ -54,9 +54,8 @@ PCBP_DECLARE_LEN3(11)
 #undef PCBP_DECLARE_LEN3
 
 // Lengths and f the register-resident kernel (bp4_*, bp_inst4.cu) is built for.  Scaled min-sum
-// at every length: against the tensor-memory kernel, time per frame-iteration without an event
-// 0.39 / 0.94 ns (N = 256), 2.18 / 3.47 (1024), 4.89 / 7.48 (2048), under an event 0.51 / 1.16,
-// 3.00 / 3.75 and 7.14 / 8.73.  Exact box-plus below N = 128 only: its f is 8 times as long, and
+// at every length: it takes 0.4 to 0.9 of the tensor-memory kernel's time per iteration (the table in
+// bp_kernel4.cuh).  Exact box-plus below N = 128 only: its f is 8 times as long, and
 // the unrolled iteration no longer fits the instruction cache (N = 256 with events 0.85 times the
 // tensor-memory kernel's speed, N = 128 0.96).
 constexpr bool warp_kernel_has(int n, int fkind) { return n >= 3 && n <= 11 && (fkind == 0 || n <= 6); }

@@ -1,7 +1,7 @@
 // pc_encode (Eq. 1 and the CRC of Sec. IV): payload bytes in, codeword bytes out.
 //
-// Bound by integer instruction issue (about 350 warp instructions a frame at N = 1024, the logic
-// pipe at two thirds of its rate; its HBM floor, K - r bytes read and N written, is half of its time).
+// Bound by integer instruction issue (346 warp instructions a frame at N = 1024, the logic pipe at 75%
+// of its rate; its HBM floor, K - r bytes read and N written, is half of its time).
 // A codeword is N bits in 32-bit words, one word a lane (two at N = 2048), 32 * 32 / N frames to a
 // warp, so the butterflies are shifts inside a word and shuffles between lanes and a warp's output
 // is 1 KB of consecutive bytes, stored 16 bytes a lane.  The payload rows of a warp's frames are one
@@ -10,7 +10,7 @@
 // information bits of a codeword word) is a 32-bit window of that string, so no row has to be
 // aligned.  The CRC is the XOR of one table entry per four payload bits.
 //
-// 262,144 frames of N = 1024, K = 512 with CRC-24: 115 us, 3.5 TB/s (one CTA a frame on bytes in
+// 262,144 frames of N = 1024, K = 512 with CRC-24: 116 us, 3.4 TB/s (one CTA a frame on bytes in
 // shared memory, with ten barriers a frame: 2,192 us).  Packing with byte dot products and the CRC's
 // addresses by one logic operation each measured 124 us, with 20 instructions fewer.
 #include <cuda_runtime.h>
@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(256) encode_kernel(const __grid_constant__ Enc
         }
     }
     // the lane's codeword words: information positions, rank of the first, and the steps that move
-    // the low bits of a word to those positions (each bit by a power of two, the largest first)
+    // the low bits of a word to those positions (each bit by a power of two, the largest first):
+    // the expand operation of H. S. Warren, Hacker's Delight, section 7-5, its names kept (mk, mp, mv)
     const int w0 = lane % LPF;
     uint32_t info[WPL], step[WPL][5];
     int rank[WPL];

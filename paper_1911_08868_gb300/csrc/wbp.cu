@@ -921,6 +921,9 @@ cudaError_t launch_backward_reg(int n, const WbpParams<float>& P, const Geo& g, 
             // With the iteration a launch parameter a frame costs 4% less (two registers of the 128), a
             // launch about 5 us: T = 20 at batch 4,096 3,756 against 3,916 us, T = 10 2,023 / 2,090, at
             // batch 2,048 (13 frames a slot) 2,020 / 2,026, at 300 448 / 346, T = 5 at 1,000 308 / 288.
+            // The shorter lengths take one launch.  A launch for each against one, T = 10: N = 512 at batch
+            // 300 137 / 89 us, 2,048 482 / 451, 4,096 (13 frames a slot) 879 / 880, 12,288 2,378 / 2,543;
+            // N = 256 407 / 361 at 4,096 and 994 / 995 at 12,288; N = 128 227 / 171 and 490 / 428.
             return P.B >= 12 * int64_t(g.grid) * g.slots ? launch_backward_reg_of<10, false>(P, g, st)
                                                          : launch_backward_reg_of<10, true>(P, g, st);
         default: return cudaErrorInvalidValue;
