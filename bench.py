@@ -453,8 +453,8 @@ def wbp_loss(logits, bits):
 WBP_ROOF_UNIT = ("per training step: stage passes S = T n + (T-1)(n-1) (the forward's L and R sweeps; the "
                  "backward recomputes them and runs their adjoints), N/2 processing elements each; lane-ops "
                  "= B S (N/2) (8 forward + 8 recomputation + 16 adjoint); HBM bytes = LLRs (forward and "
-                 "every backward launch), checkpoints written (T-1) and read (T), gradient planes between "
-                 "backward launches read and written (T-1 each), logits and their gradient")
+                 "every backward iteration), checkpoints written (T-1) and read (T), gradient planes between "
+                 "backward iterations read and written (T-1 each), logits and their gradient")
 
 
 def wbp_roofline(N, K, T, B, seconds):
