@@ -262,9 +262,12 @@ __global__ void __launch_bounds__(1024, 1) wbp_forward_reg_kernel(const __grid_c
     const bool act = tid < NH;                    // N < 64: fewer elements than a warp
     const int q = act ? tid : 0;
 
-    // every frame takes the same time: a fixed share of the frames per slot, no frame counter
+    // Every frame takes the same time: a fixed share of the frames per slot, no frame counter.  The
+    // CTAs come first in the order, then the slots, so a last round that does not fill the slots has a
+    // few frames on every SM and not many on some: batch 3,000, T = 10, N = 128 41.8 us against 56.3 the
+    // other way (47.1 with a frame counter), N = 256 85.6 / 99.4 (93.6).
     const int slots = blockDim.x / tps;
-    for (int64_t f = int64_t(blockIdx.x) * slots + slot; f < P.B; f += int64_t(gridDim.x) * slots) {
+    for (int64_t f = int64_t(slot) * gridDim.x + blockIdx.x; f < P.B; f += int64_t(gridDim.x) * slots) {
         copy_async_sw(L, P.llr + size_t(f) * N, N, tid, tps);
         for (int j = tid; j < (n - 1) * N; j += tps) R[j] = 0.f;
         if (P.ckpt)
