@@ -1,6 +1,6 @@
 // pc_encode (Eq. 1 and the CRC of Sec. IV): payload bytes in, codeword bytes out.
 //
-// Bound by integer instruction issue (346 warp instructions a frame at N = 1024, the logic pipe at 75%
+// Bound by integer instruction issue (326 warp instructions a frame at N = 1024, the logic pipe at 79%
 // of its rate; its HBM floor, K - r bytes read and N written, is half of its time).
 // A codeword is N bits in 32-bit words, one word a lane (two at N = 2048), 32 * 32 / N frames to a
 // warp, so the butterflies are shifts inside a word and shuffles between lanes and a warp's output
@@ -10,9 +10,9 @@
 // information bits of a codeword word) is a 32-bit window of that string, so no row has to be
 // aligned.  The CRC is the XOR of one table entry per four payload bits.
 //
-// 262,144 frames of N = 1024, K = 512 with CRC-24: 116 us, 3.4 TB/s (one CTA a frame on bytes in
+// 262,144 frames of N = 1024, K = 512 with CRC-24: 105 us, 3.8 TB/s (one CTA a frame on bytes in
 // shared memory, with ten barriers a frame: 2,192 us).  Packing with byte dot products and the CRC's
-// addresses by one logic operation each measured 124 us, with 20 instructions fewer.
+// addresses by one logic operation each measured 124 us against 115 at the time, with 20 instructions fewer.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,7 +40,7 @@ struct EncGeo {
     static constexpr int WARPS = 8;
     // word of contribution j while the table is made: a word in 33 left free, so that the lanes, 32
     // contributions apart, meet on no bank (one frame of N = 2048, K = 2047 23.1 -> 16.8 us, 49,157
-    // frames of K = 2046 113 -> 74)
+    // frames of K = 2046 113 -> 78)
     __host__ __device__ static constexpr int padded(int j) { return j + (j >> 5); }
     static constexpr size_t smem(int K) { return 4 * (size_t(TABLE) + std::max(WARPS * BIT_WORDS, padded(K) + 1)); }
 };
@@ -49,7 +49,9 @@ struct EncGeo {
 __device__ __forceinline__ uint32_t pack4(uint32_t b) { return ((b & 0x01010101u) * 0x01020408u) >> 24; }
 __device__ __forceinline__ uint32_t spread4(uint32_t v) { return ((v & 15u) * 0x00204081u) & 0x01010101u; }
 
-template <int LOGN>
+// WIDE: the codewords start on a 16-byte boundary and are stored 16 bytes a lane (8 below N = 32), else byte
+// by byte.  A kernel for each: with both in one, the aligned stores of N = 128 and 256 were 5% slower.
+template <int LOGN, bool WIDE>
 __global__ void __launch_bounds__(256) encode_kernel(const __grid_constant__ EncParams P)
 {
     using Geo = EncGeo<LOGN>;
@@ -107,7 +109,6 @@ __global__ void __launch_bounds__(256) encode_kernel(const __grid_constant__ Enc
     }
     __syncthreads();                                    // the table is made
     uint32_t* const bits = strings + warp * Geo::BIT_WORDS;
-    const bool wide = (reinterpret_cast<uintptr_t>(P.x) & 15u) == 0;
     const uintptr_t begin = reinterpret_cast<uintptr_t>(P.payload), end = begin + size_t(P.B) * Kp;
     // the payload of a unit as a bit string, from the 16-byte boundary at or before it: 32 bytes a
     // lane and word, read while the unit before is encoded
@@ -217,22 +218,29 @@ __global__ void __launch_bounds__(256) encode_kernel(const __grid_constant__ Enc
         if constexpr (N >= 32) {
 #pragma unroll
             for (int q = 0; q < WPL; ++q)
+                if constexpr (WIDE) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // piece 32 h + lane of 16 bytes of the warp's 1 KB
-                    const uint32_t v = __shfl_sync(0xffffffffu, x[q], 16 * h + (lane >> 1)) >> (16 * (lane & 1));
-                    const int at = 1024 * q + 512 * h + 16 * lane;
-                    if (wide && at < bytes) {
-                        __stcs(reinterpret_cast<uint4*>(out + at),
-                               make_uint4(spread4(v), spread4(v >> 4), spread4(v >> 8), spread4(v >> 12)));
-                    } else if (at < bytes) {
-#pragma unroll 1
-                        for (int b = 0; b < 16; ++b) out[at + b] = uint8_t((v >> b) & 1u);
+                    for (int h = 0; h < 2; ++h) {
+                        // piece 32 h + lane of 16 bytes of the warp's 1 KB
+                        const uint32_t v = __shfl_sync(0xffffffffu, x[q], 16 * h + (lane >> 1)) >> (16 * (lane & 1));
+                        const int at = 1024 * q + 512 * h + 16 * lane;
+                        if (at < bytes)
+                            __stcs(reinterpret_cast<uint4*>(out + at),
+                                   make_uint4(spread4(v), spread4(v >> 4), spread4(v >> 8), spread4(v >> 12)));
+                    }
+                } else {
+                    // a word at a time, a byte a lane (98,309 frames of N = 1024, K = 512 off the boundary
+                    // 65 us; with 16 bytes a lane one after another 306)
+#pragma unroll 8
+                    for (int i = 0; i < 32; ++i) {
+                        const uint32_t v = __shfl_sync(0xffffffffu, x[q], i);
+                        const int at = 1024 * q + 32 * i + lane;
+                        if (at < bytes) out[at] = uint8_t((v >> lane) & 1u);
                     }
                 }
         } else if (lane * N < bytes) {
             uint8_t* const o = out + lane * N;
-            if (wide) {
+            if constexpr (WIDE) {
 #pragma unroll
                 for (int b = 0; b < N; b += 8)
                     *reinterpret_cast<uint2*>(o + b) = make_uint2(spread4(x[0] >> b), spread4(x[0] >> (b + 4)));
@@ -254,7 +262,8 @@ int launch_encode(const EncParams& P, int sms, cudaStream_t st)
     // persistent CTAs (the table is made once per CTA; 4, 6 and 8 per SM measured alike)
     const int64_t tiles = (P.B + Geo::WARPS * Geo::FPW - 1) / (Geo::WARPS * Geo::FPW);
     const int grid = int(std::min<int64_t>(tiles, int64_t(sms) * kEncodeCtas));
-    encode_kernel<LOGN><<<grid, 256, smem, st>>>(P);
+    if ((reinterpret_cast<uintptr_t>(P.x) & 15u) == 0) encode_kernel<LOGN, true><<<grid, 256, smem, st>>>(P);
+    else encode_kernel<LOGN, false><<<grid, 256, smem, st>>>(P);
     return cudaGetLastError() == cudaSuccess ? PC_OK : PC_ECUDA;
 }
 
