@@ -321,12 +321,20 @@ int plan_launch4(const pc_code* c, int64_t B, LaunchGeom* g, int slots_req = 0)
     slots = int(std::max<int64_t>(1, std::min<int64_t>(slots, (B + di.sms - 1) / di.sms)));
     int max_slots = 0;
     shape4_of(c->n, c->K, slots, &max_slots, &smem);
-    // over half of an SM's shared memory: one CTA per SM, so the tensor-memory allocation never waits
-    smem = std::max(smem, size_t(di.smem_per_sm) / 2 + 1024);
+    // Below N = 128 a request for fewer frames per CTA than fit leaves the SM's other warps to more CTAs.
+    // 50,000 frames of N = 16 at one frame per CTA 48 us, with one CTA per SM 315 (75 with the
+    // shared-memory kernel); N = 64 965, 6,738 (3,317).
+    const int ctas = c->n < 7 && slots == slots_req ? std::max(1, std::min(kShortCtas, max_slots / slots)) : 1;
+    // Shared memory beyond an SM's 1 / (ctas + 1), so no more CTAs than that per SM (each takes 1 KB more
+    // than it asks for) and no tensor-memory allocation waits for a CTA of this launch; one CTA asks for
+    // over half, so its allocation never waits.
+    const size_t share = ctas > 1 ? (size_t(di.smem_per_sm) / ctas & ~size_t(1023)) - 1152
+                                  : size_t(di.smem_per_sm) / 2 + 1024;
+    smem = std::max(smem, share);
     if (smem > size_t(di.smem_optin)) return PC_EUNSUPPORTED;
     g->slots = slots;
     g->smem = smem;
-    g->grid = int(std::min<int64_t>((B + slots - 1) / slots, di.sms));
+    g->grid = int(std::min<int64_t>((B + slots - 1) / slots, int64_t(di.sms) * ctas));
     return PC_OK;
 }
 

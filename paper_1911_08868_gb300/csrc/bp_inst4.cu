@@ -15,6 +15,7 @@ namespace pcbp {
 
 namespace {
 using Geo = G4<PCBP_LOGN>;
+static_assert(PCBP_LOGN >= 7 || kShortCtas * Geo::tm_cols() <= 512, "no allocation waits for a CTA of its launch");
 
 // pdl: programmatic dependent launch, the grid may start while the previous
 // kernel of the stream still runs (for independent batches).

@@ -62,6 +62,9 @@ constexpr bool warp_kernel_has(int n, int fkind) { return n >= 3 && n <= 11 && (
 
 struct WarpParams;
 
+// CTAs of the register-resident kernel that an SM's tensor memory holds at once below N = 128.
+constexpr int kShortCtas = 8;
+
 #define PCBP_DECLARE_LEN4(n)                                                                       \
     void bp4_shape_##n(int K, int slots, int* max_slots_out, size_t* smem_out);                    \
     cudaError_t bp4_launch_##n(const WarpParams& P, const LaunchGeom& g, int fkind, cudaStream_t st, bool pdl); \
